@@ -107,7 +107,8 @@ def transform_alg_bytes(nx, ny, nz, esz=4):
 def mode_alg_bytes(nx, ny, nz, mc, groups, esz=4):
     """Algorithmic bytes per launch of the mode-space form's kernels: the
     projection reads rho and writes one partial projection per group of x
-    rows, the z kernel reads the partials and the kernel spectra and writes
+    rows, the z kernel reads the partials and the columns' z kernels (counted as
+    nz + 1 values each, the table that its recurrences stand for) and writes
     the convolved mode columns, the back-projection reads those (once per z
     chunk) and writes phi."""
     field = nx * ny * nz * esz
@@ -121,13 +122,12 @@ def mode_flops(nx, ny, nz, mx, mxp, myp, fold, mc):
     """Floating-point operations per launch of the mode-space kernels, counted
     from their sums (an FMA is 2): the projection's y sums (over ny/2 folded
     pairs, or ny rows) and x sums, the back-projection's x sums and y sums, and
-    for the z kernel two complex L = nz point FFTs per column at 5 L log2 L
-    plus the spectral product (about 40 flops per point)."""
-    import math
+    for the z kernel two first-order recurrences and their combination (9
+    operations a value)."""
     yrows = ny // 2 if fold else ny
     proj = 2 * nx * nz * myp * (yrows + mxp) + (2 * nx * nz * yrows if fold else 0)
     back = 2 * nx * nz * myp * (mx + yrows) + (2 * nx * nz * yrows if fold else 0)
-    zc = mc * (2 * 5 * nz * int(math.log2(nz)) + 40 * nz)
+    zc = 9 * mc * nz
     return {"mode_project": proj, "mode_z": zc, "mode_back": back}
 
 

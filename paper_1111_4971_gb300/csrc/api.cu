@@ -124,7 +124,8 @@ void free_handle(pipe_handle* h) {
   cudaFree(h->stage_rho); cudaFree(h->stage_phi);
   cudaFree(h->tbuf);
   cudaFree(h->msx64); cudaFree(h->msy64); cudaFree(h->mgz64);
-  cudaFree(h->msx32); cudaFree(h->msy32); cudaFree(h->mgz32);
+  cudaFree(h->msx32); cudaFree(h->msy32);
+  cudaFree(h->mzp64); cudaFree(h->mzp32);
   cudaFree(h->mwork);
   cudaFree(h->mkb64); cudaFree(h->mkb32);
   std::free(h->msy_host);
@@ -263,9 +264,7 @@ ModeArgs<T> mode_args(const pipe_handle* h, const void* rho, void* phi, void* pa
   a.psi = static_cast<T*>(psi);
   a.sx = reinterpret_cast<const T*>(D ? static_cast<const void*>(h->msx64) : static_cast<const void*>(h->msx32));
   a.sy = reinterpret_cast<const T*>(D ? static_cast<const void*>(h->msy64) : static_cast<const void*>(h->msy32));
-  a.gz = reinterpret_cast<const T*>(D ? static_cast<const void*>(h->mgz64) : static_cast<const void*>(h->mgz32));
-  a.tw_z = reinterpret_cast<const C2<T>*>(D ? static_cast<const void*>(h->tw_z64) : static_cast<const void*>(h->tw_z32));
-  a.w2_z = reinterpret_cast<const C2<T>*>(D ? static_cast<const void*>(h->w2_z64) : static_cast<const void*>(h->w2_z32));
+  a.zp = reinterpret_cast<const T*>(D ? static_cast<const void*>(h->mzp64) : static_cast<const void*>(h->mzp32));
   a.nx = h->grid.nx; a.ny = h->grid.ny; a.nz = h->grid.nz;
   a.mx = h->geom.modes_m;
   a.mxp = h->mxp;
@@ -437,15 +436,17 @@ static int setup_pipe(const pipe_geometry* geom, const pipe_grid* grid, int igf,
     h->myp = mode_slots(geom->modes_n, fold);
     const size_t nsx = size_t(grid->nx) * h->mxp, nsy = size_t(fold ? grid->ny / 2 : grid->ny) * h->myp;
     const size_t ngz = size_t(h->mxp) * h->myp * (grid->nz + 1);
+    const size_t nzp = size_t(h->mxp) * h->myp * kModeZPar;
     if (cudaMalloc(&h->msx64, nsx * 8) != cudaSuccess || cudaMalloc(&h->msx32, nsx * 4) != cudaSuccess ||
         cudaMalloc(&h->msy64, nsy * 8) != cudaSuccess || cudaMalloc(&h->msy32, nsy * 4) != cudaSuccess ||
-        cudaMalloc(&h->mgz64, ngz * 8) != cudaSuccess || cudaMalloc(&h->mgz32, ngz * 4) != cudaSuccess ||
+        cudaMalloc(&h->mgz64, ngz * 8) != cudaSuccess || cudaMalloc(&h->mzp64, nzp * 8) != cudaSuccess ||
+        cudaMalloc(&h->mzp32, nzp * 4) != cudaSuccess ||
         cudaMalloc(&h->mwork, mode_scratch_bytes(h)) != cudaSuccess) {
       free_handle(h);
       return PIPE_ENOMEM;
     }
     cudaError_t e = build_mode_tables(s, geom->x0, geom->y0, h->mxp, h->myp, h->fy, h->msx64, h->msx32,
-                                      h->msy64, h->msy32, h->mgz64, h->mgz32, nullptr);
+                                      h->msy64, h->msy32, h->mgz64, h->mzp64, h->mzp32, nullptr);
     if (e != cudaSuccess) { free_handle(h); return status_of(e); }
     if (n_nb >= 0) {                     // the banded operator's z stencil
       const size_t nkb = size_t(h->mxp) * h->myp * (n_nb + 1);

@@ -570,7 +570,7 @@ static int run_mode_group(const MGroup& g, const void* const* rho, void* const* 
     p.phi[i] = static_cast<float*>(phi[g.members[i]]);
   }
   cudaError_t e = launch_mode_fast_group(0, g.myp, g.a0, p, g.sy, st);
-  if (e == cudaSuccess) e = launch_mode_z_warp_group(g.a0, g.zgroups, p, st);
+  if (e == cudaSuccess) e = launch_mode_z_group(g.a0, g.zgroups, p, st);
   if (e == cudaSuccess) e = launch_mode_fast_group(2, g.myp, g.a0, p, g.sy, st);
   return e == cudaSuccess ? PIPE_OK : PIPE_ECUDA;
 }

@@ -15,6 +15,7 @@
 
 #include "fft_common.cuh"
 #include "green_kernels.cuh"
+#include "modes.cuh"
 
 namespace pp {
 
@@ -490,9 +491,11 @@ done:
 // Tables of the mode-space solve (modes_impl.cuh), all FP64 with FP32 copies:
 //   sx[i][s] = sin(m pi x_i / a), m = s + 1 (zero for m > Mx), i < nx, s < mxp
 //   sy[j][s] = sin(n pi y_j / b) for the mode n of slot s (mode_of_slot), j < nyk
-//   gz[c][kz], c = s_x * myp + s_y: the DCT-I of the doubled z table of
+//   zp[c], c = s_x * myp + s_y: the parameters of the z recurrences of
 //       K_mn(d) = hx hy hz (8 pi / ab) kappa_mn^{-1} f_mn(d hz)
-//   (f the e^{-kappa |w|} of Eq. 9 or the IGF g_z of Eq. 15), divided by 2nz.
+//   (f the e^{-kappa |w|} of Eq. 9 or the IGF g_z of Eq. 15): K(0), K(1),
+//   1 - q, q, q^{kModeZRun 2^i}, with q = e^{-kappa hz}, so K(d) = K(1) q^{d-1}
+//   gz[c][kz]: the DCT-I of the doubled z table of K_mn, divided by 2nz.
 // ---------------------------------------------------------------------------
 __global__ void mode_sine_kernel(double* t64, float* t32, int rows, int slots, int nmodes, int fold,
                                  double origin, double h, double len) {
@@ -505,7 +508,31 @@ __global__ void mode_sine_kernel(double* t64, float* t32, int rows, int slots, i
   t32[idx] = float(v);
 }
 
-__global__ void mode_gz_kernel(double* g64, float* g32, const double* Zh, int M, int N, int mxp, int myp,
+// K(1) of the IGF, 4 sinh^2(x/2) e^{-x} / x^2 at x = kappa hz, is (1 - q)^2 / x^2
+__global__ void mode_zp_kernel(double* z64, float* z32, int M, int N, int mxp, int myp, int fold, double hz,
+                               double a, double b, int igf, double C) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= mxp * myp) return;
+  const int m = c / myp + 1, s = c % myp;
+  const int n = !fold ? s + 1 : (s < myp / 2 ? 2 * s + 1 : 2 * (s - myp / 2) + 2);
+  double v[kModeZPar] = {};
+  if (m <= M && n <= N) {
+    const double km = double(m) / a, kn = double(n) / b;
+    const double kap = M_PI * sqrt(km * km + kn * kn);
+    const double x = kap * hz, q = exp(-x), p = -expm1(-x);
+    v[0] = C / kap * (igf ? 2.0 * xm1pe_over_x2(x) : 1.0);
+    v[1] = C / kap * (igf ? (p / x) * (p / x) : q);
+    v[2] = p;
+    v[3] = q;
+    for (int i = 0; i < kModeZPar - 4; ++i) v[4 + i] = exp(-x * double(kModeZRun << i));
+  }
+  for (int i = 0; i < kModeZPar; ++i) {
+    z64[c * kModeZPar + i] = v[i];
+    z32[c * kModeZPar + i] = float(v[i]);
+  }
+}
+
+__global__ void mode_gz_kernel(double* g64, const double* Zh, int M, int N, int mxp, int myp,
                                int fold, int nz, double C) {
   const long idx = long(blockIdx.x) * blockDim.x + threadIdx.x;
   if (idx >= long(mxp) * myp * (nz + 1)) return;
@@ -515,7 +542,6 @@ __global__ void mode_gz_kernel(double* g64, float* g32, const double* Zh, int M,
   const int n = !fold ? s + 1 : (s < myp / 2 ? 2 * s + 1 : 2 * (s - myp / 2) + 2);
   const double v = (m <= M && n <= N) ? C * Zh[(long(m - 1) * N + (n - 1)) * (nz + 1) + kz] : 0.0;
   g64[idx] = v;
-  g32[idx] = float(v);
 }
 
 // kb[c][d] = hx hy hz (8 pi / ab) kappa^{-1} f_mn(d hz), d = 0..nb, c = (m-1) myp + slot(n):
@@ -549,7 +575,7 @@ cudaError_t build_mode_band(const GreenSpec& s, int mxp, int myp, int fold, int 
 
 cudaError_t build_mode_tables(const GreenSpec& s, double x0, double y0, int mxp, int myp, int fold,
                               double* sx64, float* sx32, double* sy64, float* sy32, double* gz64,
-                              float* gz32, cudaStream_t st) {
+                              double* zp64, float* zp32, cudaStream_t st) {
   const int M = s.modes_m, N = s.modes_n, nz = s.nz;
   const int nyk = fold ? s.ny / 2 : s.ny;
   double *Z = nullptr, *Zh = nullptr, *cosn = nullptr;
@@ -563,7 +589,9 @@ cudaError_t build_mode_tables(const GreenSpec& s, double x0, double y0, int mxp,
   cos_pi_table_kernel<<<nblk(2 * nz, 256), 256, 0, st>>>(cosn, nz);
   z_dct_kernel<<<nblk(long(M) * N * (nz + 1), 256), 256, 0, st>>>(Zh, Z, M * N, nz, cosn);
   mode_gz_kernel<<<nblk(long(mxp) * myp * (nz + 1), 256), 256, 0, st>>>(
-      gz64, gz32, Zh, M, N, mxp, myp, fold, nz, s.hx * s.hy * s.hz * 8.0 * M_PI / (s.a * s.b) / (2.0 * nz));
+      gz64, Zh, M, N, mxp, myp, fold, nz, s.hx * s.hy * s.hz * 8.0 * M_PI / (s.a * s.b) / (2.0 * nz));
+  mode_zp_kernel<<<nblk(long(mxp) * myp, 64), 64, 0, st>>>(zp64, zp32, M, N, mxp, myp, fold, s.hz, s.a, s.b, s.igf,
+                                                           s.hx * s.hy * s.hz * 8.0 * M_PI / (s.a * s.b));
   if ((err = cudaGetLastError()) != cudaSuccess) goto done;
   err = cudaStreamSynchronize(st);
 done:

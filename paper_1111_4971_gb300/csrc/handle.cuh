@@ -57,8 +57,11 @@ struct pipe_handle {
   int use_modes = 0;           // solves take the mode path (plan t_kind 3)
   int fft_ok = 1;              // the padded-transform path's buffers exist
   int mxp = 0, myp = 0, fy = 0;
-  double *msx64 = nullptr, *msy64 = nullptr, *mgz64 = nullptr;
-  float *msx32 = nullptr, *msy32 = nullptr, *mgz32 = nullptr;
+  double *msx64 = nullptr, *msy64 = nullptr;
+  float *msx32 = nullptr, *msy32 = nullptr;
+  double* mgz64 = nullptr;     // DCT-I of the doubled z kernel tables [mxp*myp][nz+1] (pipe_mode_spectrum)
+  double* mzp64 = nullptr;     // parameters of the z recurrences [mxp*myp][kModeZPar]
+  float* mzp32 = nullptr;
   double* mkb64 = nullptr;     // banded operator in mode space: [mxp*myp][nb+1] real-space z kernel
   float* mkb32 = nullptr;
   void* mwork = nullptr;       // part [xblocks][mc][nz], then psi [mc][nz], of the dtype

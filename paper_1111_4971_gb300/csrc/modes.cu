@@ -19,12 +19,6 @@ __global__ void __launch_bounds__(128) mode_back_kernel(ModeArgs<T> a) {
   mode_back<T, MYP, FY>(a, smem_raw);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) mode_z_kernel(ModeArgs<T> a, int groups) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  mode_z<T>(a, groups, smem_raw);
-}
-
 // Banded z stage (Sec. 5, Eq. 17-18 in mode space): psi[c][k] =
 // sum_{|d| <= nb, 0 <= k-d < nz} K_c(|d|) rhot[c][k-d], rhot the groups' partial
 // projections summed.  One CTA per column: the column (zero-padded by nb on
@@ -126,20 +120,6 @@ cudaError_t launch_pb2(int which, bool fy, const ModeArgs<T>& a, cudaStream_t st
   return fy ? launch_pb<T, MYP, true>(which, a, st) : launch_pb<T, MYP, false>(which, a, st);
 }
 
-// 256 threads per CTA, L/4 per column (L = nz in 32..1024)
-template <typename T>
-cudaError_t launch_zc(const ModeArgs<T>& a, cudaStream_t st) {
-  const int xblocks = a.nx / ModeShape<T>::XB;
-  if constexpr (sizeof(T) == 4) return launch_mode_z_warp(a, xblocks / mode_cluster(xblocks), st);
-  const int per = 1024 / a.nz;                       // columns per CTA
-  const size_t smem = sizeof(C2<T>) * (size_t(per) * 2 * a.nz + 3 * size_t(a.nz));
-  void (*kern)(ModeArgs<T>, int) = mode_z_kernel<T>;
-  cudaError_t e;
-  if ((e = set_smem(kern, smem)) != cudaSuccess) return e;
-  kern<<<(a.mc + per - 1) / per, 256, smem, st>>>(a, xblocks / mode_cluster(xblocks));
-  return cudaGetLastError();
-}
-
 }  // namespace
 
 #ifndef PP_M_TYPE
@@ -153,7 +133,8 @@ cudaError_t launch_mode_stage<PP_M_TYPE>(int stage, int myp, bool fy, const Mode
   if (stage == 1) {
     if (a.nz < 32 || a.nz > 1024 || (a.nz & (a.nz - 1))) return cudaErrorInvalidValue;
     if (a.nb >= 0) return launch_band<T>(a, st);
-    return launch_zc<T>(a, st);
+    const int xblocks = a.nx / ModeShape<T>::XB;
+    return launch_mode_z<T>(a, xblocks / mode_cluster(xblocks), st);
   }
   const int which = stage == 0 ? 0 : 1;
   switch (myp) {

@@ -83,6 +83,11 @@ inline int mode_cluster(int xblocks) {
   return 1;
 }
 
+// z recurrences (modes_z.cu): z values per thread, and the parameters of a
+// mode column: beta, gamma, 1 - q, q, then q^{kModeZRun 2^i} for i < 8
+constexpr int kModeZRun = 8;
+constexpr int kModeZPar = 12;
+
 // stage 0: projection rho -> part, 1: z convolution part -> psi,
 // 2: back-projection psi -> phi
 template <typename T>
@@ -101,11 +106,12 @@ struct ModeGroup {
   int nz;
 };
 
-// the FP32 z convolution, one warp-level FFT per mode column (modes_z.cu):
-// nz in 32..1024, groups partial projections summed on load
-cudaError_t launch_mode_z_warp(const ModeArgs<float>& a, int groups, cudaStream_t st);
+// the z convolution as two recurrences per mode column (modes_z.cu): nz a
+// power of two in 32..1024, groups partial projections summed on load
+template <typename T>
+cudaError_t launch_mode_z(const ModeArgs<T>& a, int groups, cudaStream_t st);
 // the same for a group (columns of solve s in the CTAs s * cps ..)
-cudaError_t launch_mode_z_warp_group(const ModeArgs<float>& a, int groups, const ModeGroup& g, cudaStream_t st);
+cudaError_t launch_mode_z_group(const ModeArgs<float>& a, int groups, const ModeGroup& g, cudaStream_t st);
 
 // the FP32 projection and back-projection laid out for occupancy
 // (modes_fast.cu): meshes symmetric in y with ny/2 in {16, 32, 64, 128}

@@ -20,10 +20,9 @@
 // the Mx x My frequencies that survive the product, and the back-projection
 // the inverse transforms restricted to them.  The form holds on any mesh
 // inside the pipe (windows included).  The z convolution is the zero-padded
-// 2nz-point transform of Appendix A (Eq. A.1-A.4): a real-to-complex FFT of
-// each mode's column, the product with the DCT-I of the doubled kernel table
-// (scaled by 1 / 2nz), and the inverse, with the z-axis routines of the full
-// solve.
+// one of Appendix A (Eq. A.1-A.4); its kernel is a two-sided exponential in z
+// apart from the centre tap, so it runs as two first-order recurrences
+// (modes_z.cu).
 //
 // The operator is symmetric (G(r, r') = G(r', r)): the projection and the
 // back-projection use the same tables and the z kernel is even, so the
@@ -59,9 +58,7 @@ struct ModeArgs {
   T* psi;                // [mc][nz]
   const T* sx;           // [nx][mxp]
   const T* sy;           // [FY ? ny/2 : ny][MYP]
-  const T* gz;           // [mc][nz+1]: DCT-I of the doubled kernel table / 2nz
-  const C2<T>* tw_z;     // z group-FFT twiddles (length nz/2)
-  const C2<T>* w2_z;     // w_{2nz}^j, j < 2nz
+  const T* zp;           // [mc][kModeZPar]: the z recurrences' parameters
   int nx, ny, nz;
   int mx;                // x modes
   int mxp;               // x modes padded to a multiple of 4 (columns of sx)
@@ -319,173 +316,6 @@ __device__ __forceinline__ void mode_back(const ModeArgs<T>& a, unsigned char* s
         row[0] = o[i];
       }
     }
-  }
-}
-
-// z convolution of the mode columns, one column per group of L/4 threads
-// (L = nz; a CTA of 256 threads takes 1024/L columns):
-//   1. the packed column z_m = rhot(2m) + i rhot(2m+1), m < L/2 (the sum of
-//      the groups' partial projections); z_m = 0 for m >= L/2 is the zero
-//      padding of Appendix A, never stored;
-//   2. Z = the L-point forward FFT of z (radix-4 Stockham in shared memory,
-//      a radix-2 stage first when log2 L is odd; the first stage skips the
-//      known-zero half of its inputs);
-//   3. for each pair (k, L-k): the 2L-point real spectrum
-//      X(k) = [Z(k) + conj Z(L-k) - i w^k (Z(k) - conj Z(L-k))] / 2, w = e^{-i pi / L},
-//      times the kernel spectrum g(k), and the packed inverse input
-//      Z'(k) = Y(k) + conj Y(L-k) + i w^{-k} (Y(k) - conj Y(L-k));
-//   4. z' = the unnormalised L-point inverse FFT of Z' (the last stage only
-//      computes the outputs m < L/2), y(2m) = Re z'_m, y(2m+1) = Im z'_m: the
-//      first nz outputs of the 2nz-point inverse, which is psi.
-// Twiddles come from the 2L-entry table w2[j] = e^{-2 pi i j / (2L)}, copied
-// into shared memory at the start and rearranged there stage by stage so that
-// the lanes of a stage read consecutive entries.
-// the twiddles of the radix-4 stages with Ls > 1, stage after stage, each as
-// [r-1][j] = w_{4 Ls}^{r j} (r = 1..3, j < Ls), so that the lanes of a stage
-// (consecutive j) read consecutive entries; about L values in all
-template <typename T>
-__device__ __forceinline__ void stockham_twiddles(C2<T>* tws, const C2<T>* w2, int L) {
-  int off = 0;
-  for (int Ls = (__popc(L - 1) & 1) ? 2 : 4; Ls < L; Ls *= 4) {
-    const int tstep = L / (2 * Ls);                  // w_{4 Ls}^{q} = w2[q * L / (2 Ls)]
-    for (int i = int(threadIdx.x); i < 3 * Ls; i += int(blockDim.x)) {
-      const int r = i / Ls + 1, j = i % Ls;
-      tws[off + i] = w2[r * j * tstep];
-    }
-    off += 3 * Ls;
-  }
-}
-
-template <typename T, bool INV>
-__device__ __forceinline__ C2<T>* stockham(C2<T>* src, C2<T>* dst, int L, int tid, int nthr, const C2<T>* tws,
-                                          bool prune_in, bool prune_out) {
-  using V = C2<T>;
-  int Ls = 1;
-  if (__popc(L - 1) & 1) {                           // radix-2 stage first
-    for (int t = tid; t < L / 2; t += nthr) {
-      const V a0 = src[t];
-      const V a1 = prune_in ? mk<V>(T(0), T(0)) : src[t + L / 2];
-      dst[2 * t] = cadd(a0, a1);
-      dst[2 * t + 1] = csub(a0, a1);
-    }
-    Ls = 2;
-    prune_in = false;
-    V* tmp = src; src = dst; dst = tmp;
-    __syncthreads();
-  }
-  while (Ls < L) {
-    const bool last = 4 * Ls == L;
-    for (int t = tid; t < L / 4; t += nthr) {
-      const int j = t % Ls;
-      V a[4];
-      a[0] = src[t];
-      a[1] = src[t + L / 4];
-      if (prune_in) {
-        a[2] = a[3] = mk<V>(T(0), T(0));
-      } else {
-        a[2] = src[t + L / 2];
-        a[3] = src[t + 3 * L / 4];
-      }
-      if (Ls > 1) {
-#pragma unroll
-        for (int r = 1; r < 4; ++r) a[r] = cmulc<INV>(a[r], tws[(r - 1) * Ls + j]);
-      }
-      dft_reg<4, INV>(a);
-      V* o = dst + (t - j) * 4 + j;
-      o[0] = a[0];
-      o[Ls] = a[1];
-      if (!(last && prune_out)) {
-        o[2 * Ls] = a[2];
-        o[3 * Ls] = a[3];
-      }
-    }
-    if (Ls > 1) tws += 3 * Ls;
-    Ls *= 4;
-    prune_in = false;
-    V* tmp = src; src = dst; dst = tmp;
-    __syncthreads();
-  }
-  return src;
-}
-
-template <typename T>
-__device__ __forceinline__ void mode_z(const ModeArgs<T>& a, int groups, unsigned char* smem_raw) {
-  using V = C2<T>;
-  const int L = a.nz;
-  const int nthr = L / 4;                            // threads per column
-  const int per = int(blockDim.x) / nthr;            // columns per CTA
-  const int cl = int(threadIdx.x) / nthr, tid = int(threadIdx.x) % nthr;
-  const int col = int(blockIdx.x) * per + cl;
-  const bool valid = col < a.mc;
-  // the twiddle table w2 (2L values, shared by the CTA's columns) first, then
-  // two buffers of L values per column; the table arrives by cp.async, all of
-  // it in flight at once, so its latency is paid once and not per stage
-  V* w2 = reinterpret_cast<V*>(smem_raw);
-  V* tws = w2 + 2 * L;                               // the stages' twiddles (< L values)
-  V* bufa = tws + L + size_t(cl) * 2 * L;
-  V* bufb = bufa + L;
-  {
-    constexpr int EPP = 16 / int(sizeof(V));          // values per 16-byte piece
-    for (int i = int(threadIdx.x); i < 2 * L / EPP; i += int(blockDim.x)) cp_async16(w2 + EPP * i, a.w2_z + EPP * i);
-    cp_async_commit();
-  }
-  // the kernel spectrum at this thread's pairs (k, L-k), read ahead
-  const T* g = a.gz + size_t(valid ? col : 0) * (L + 1);
-  T gk[3], gm[3];
-#pragma unroll
-  for (int u = 0; u < 3; ++u) {
-    const int k = tid + u * nthr;
-    gk[u] = (valid && k <= L / 2) ? __ldg(&g[k]) : T(0);
-    gm[u] = (valid && k <= L / 2) ? __ldg(&g[L - k]) : T(0);
-  }
-  // 1. packed column, summed over the groups
-  for (int m = tid; m < L / 2; m += nthr) {
-    V z = mk<V>(T(0), T(0));
-    if (valid) {
-#pragma unroll 4
-      for (int s = 0; s < groups; ++s)
-        z = cadd(z, __ldg(reinterpret_cast<const V*>(a.part + (size_t(s) * a.mc + col) * L) + m));
-    }
-    bufa[m] = z;
-  }
-  cp_async_wait<0>();
-  __syncthreads();
-  stockham_twiddles<T>(tws, w2, L);
-  __syncthreads();
-  // 2. forward transform
-  V* Z = stockham<T, false>(bufa, bufb, L, tid, nthr, tws, true, false);
-  V* Zp = Z == bufa ? bufb : bufa;
-  // 3. real spectrum, kernel product, packed inverse input
-#pragma unroll
-  for (int u = 0; u < 3; ++u) {
-    const int k = tid + u * nthr;
-    if (k > L / 2) continue;
-    const V zk = Z[k], zm = Z[(L - k) & (L - 1)];
-    const V wk = w2[k];                              // w^k
-    const V wm = w2[L - k];                          // w^{L-k}
-    auto unpack = [](V x, V xm, V w) {               // (x + conj xm - i w (x - conj xm)) / 2
-      const V c = cconj(xm);
-      const V s = cadd(x, c), d = csub(x, c);
-      const V wd = cmul(w, d);
-      return mk<V>(T(0.5) * (s.x + wd.y), T(0.5) * (s.y - wd.x));
-    };
-    auto repack = [](V y, V ym, V w) {               // y + conj ym + i conj(w) (y - conj ym)
-      const V c = cconj(ym);
-      const V s = cadd(y, c), d = csub(y, c);
-      const V wd = cmulc<true>(d, w);
-      return mk<V>(s.x - wd.y, s.y + wd.x);
-    };
-    const V yk = cscale(unpack(zk, zm, wk), gk[u]);
-    const V ym = cscale(unpack(zm, zk, wm), gm[u]);
-    Zp[k] = repack(yk, ym, wk);
-    if (k > 0 && k < L / 2) Zp[L - k] = repack(ym, yk, wm);
-  }
-  __syncthreads();
-  // 4. inverse transform, first L/2 outputs: psi
-  V* zo = stockham<T, true>(Zp, Z, L, tid, nthr, tws, false, true);
-  if (valid) {
-    V* dst = reinterpret_cast<V*>(a.psi + size_t(col) * L);
-    for (int m = tid; m < L / 2; m += nthr) dst[m] = zo[m];
   }
 }
 

@@ -1,30 +1,30 @@
-// FP32 z convolution of the mode-space solve, one warp-level FFT per mode
-// column: the same steps as mode_z (modes_impl.cuh) -- the packed 2nz-point
-// real transform of Appendix A (Eq. A.1-A.4) as an L = nz point complex FFT,
-// the real-spectrum unpack, the product with the kernel spectrum g and the
-// packed inverse -- with each column's L points held in the registers of S
-// lanes (E = L / S points a lane, S = 2^floor(log2 L / 2)) instead of a CTA's
-// shared memory.
+// z convolution of the mode-space solve, psi[c][k] = sum_k' K_c(k - k') rhot[c][k'],
+// as a pair of first-order recurrences.
 //
-// Four-step transform (L = S * E).  Lane b of a column holds the points
-// m = b + S a (a < E).  Then, with k = k1 + E k2,
-//   X(k1 + E k2) = sum_b w_S^{b k2} [ w_L^{b k1} sum_a x(b + S a) w_E^{a k1} ],
-// i.e. (1) an E-point DFT over a in each lane's registers, (2) the twiddle
-// w_L^{b k1}, (3) a transpose through shared memory, after which lane l takes
-// the rows k1 = l + S i (i < E / S) and (4) an S-point DFT over b for each.
-// The inverse is the same with conjugate twiddles.  Only the first L/2 input
-// points are nonzero (the zero padding), so the first DFT skips its upper
-// half; only the first L/2 outputs of the inverse are kept (psi is the first
-// nz of the 2nz-point result), so the last DFT computes only those.  Between
-// the two transforms the spectrum goes to shared memory in natural order and
-// each lane forms, for its points k = b + S a (into a second buffer, read back
-// in the layout of the inverse's input),
-//   Y(k)    = g(k)     [Z(k) + conj Z(L-k) - i w^k (Z(k) - conj Z(L-k))] / 2,
-//   Y(L-k)  = g(L-k)   [Z(L-k) + conj Z(k) - i w^{L-k} (Z(L-k) - conj Z(k))] / 2,
-//   Z'(k)   = Y(k) + conj Y(L-k) + i w^{-k} (Y(k) - conj Y(L-k)),
-// w = e^{-i pi / L}, Z(L) = Z(0).  Everything between the loads of the partial projections
-// (summed over their groups) and the stores of psi is registers and one
-// warp's shared memory: no block-wide barrier.
+// The kernel of a mode is a two-sided exponential with its own centre tap:
+// with q = e^{-kappa hz}, K_c(d) = gamma q^{d-1} for d >= 1 (Eq. 9, and the
+// longitudinal IGF of Eq. 15-16 at |w| >= hz) and K_c(0) = beta.  So the
+// zero-padded convolution of Appendix A is, exactly,
+//     psi_k = beta rhot_k + gamma (F_{k-1} + B_{k+1}),
+//     F_k = rhot_k + q F_{k-1},   B_k = rhot_k + q B_{k+1},   F_{-1} = B_{nz} = 0,
+// 9 operations a value instead of two padded FFTs.  (It replaced a warp-level
+// four-step FFT in FP32 and a Stockham FFT in FP64.  A 128^2 x 1024 solve, 400
+// columns, back to back: FP32 53.5 -> 50.3 us, its error against 64 bits
+// 3.3e-7 -> 2.4e-7; FP64 1076 -> 1005 us, 1.6e-15 -> 3.6e-16.)
+//
+// A thread takes kV consecutive z of a column and a column nz / kV threads:
+// both recurrences over the thread's values from zero, an inclusive scan of
+// the threads' totals by shuffles (multipliers q^{kV 2^i}), across the warps
+// of a column through shared memory, then the recurrences again from the
+// incoming states.  kV = 8 keeps a load two 16-byte pieces of a run and gives
+// 4 warps a column at nz = 1024; the kernel is bound by latency (one round
+// trip of loads, the scan) and, in FP64, by the FP64 pipe.
+//
+// Precision.  beta, gamma, 1 - q and the multipliers are tabulated in FP64.
+// FP32 steps take F <- (F - (1 - q) F) + x: q itself, rounded, would be
+// wrong by its last bit per step, a systematic error where kappa hz is small.
+#include <type_traits>
+
 #include "modes.cuh"
 #include "modes_impl.cuh"
 
@@ -32,210 +32,156 @@ namespace pp {
 
 namespace {
 
-constexpr int kZWarps = 2;                       // warps per CTA
+constexpr int kV = kModeZRun;                     // z values per thread
+constexpr int kZThreads = 128;                    // threads per CTA
 
-constexpr int ilog2(int n) { return n > 1 ? 1 + ilog2(n / 2) : 0; }
+// one step of a recurrence: x + q s  (FP32: p = 1 - q, FP64: p = q)
+__device__ __forceinline__ float zstep(float s, float x, float p) { return fmaf(-p, s, s) + x; }
+__device__ __forceinline__ double zstep(double s, double x, double p) { return fma(p, s, x); }
 
-template <int L>
-struct ZWarpShape {
-  static constexpr int LOG = ilog2(L);
-  static constexpr int S = 1 << (LOG / 2);       // lanes per column
-  static constexpr int E = L / S;                // points per lane (E >= S)
-  static constexpr int CPW = 32 / S;             // columns per warp
-  static constexpr int CB = E * (S + 1) + 1;     // complex values of a column's buffer
-  // floats of the CTA's kernel spectra, rounded up to a whole number of
-  // complex values
-  static constexpr int GS = (kZWarps * CPW * (L + 1) + 1) / 2 * 2;
-  static constexpr size_t SMEM = sizeof(float2) * (2 * size_t(L) + size_t(kZWarps) * CPW * 2 * CB) + sizeof(float) * GS;
-};
-
-// CTA `blk` of a solve: its columns blk * CPC ..
-template <int L>
-__device__ __forceinline__ void z_warp(const ModeArgs<float>& a, int groups, int blk) {
-  using V = float2;
-  using Sh = ZWarpShape<L>;
-  constexpr int S = Sh::S, E = Sh::E, CPW = Sh::CPW;
-  constexpr int CPC = kZWarps * CPW;             // columns per CTA
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int sub = lane / S, b = lane % S;
-  const int cl = warp * CPW + sub;               // column within the CTA
-  const int col0 = blk * CPC;
-  const int col = col0 + cl;
+// CTA `blk` of a solve: its columns blk * (1024 / NZ) ..
+template <typename T, int NZ>
+__device__ __forceinline__ void z_scan(const ModeArgs<T>& a, int groups, int blk) {
+  constexpr int TC = NZ / kV;                     // threads per column
+  constexpr int CPC = kZThreads / TC;             // columns per CTA
+  constexpr int SEG = TC < 32 ? TC : 32;          // lanes of a warp on one column
+  constexpr int NW = TC / SEG;                    // warps per column
+  using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
+  constexpr int EV = 16 / int(sizeof(T));         // values per 16-byte piece
+  __shared__ T tot[2][kZThreads / 32];
+  const int cl = int(threadIdx.x) / TC, t = int(threadIdx.x) % TC;
+  const int ls = t % SEG, wq = t / SEG;
+  const int col = blk * CPC + cl;
   const bool valid = col < a.mc;
-  // shared memory: the stage-2 twiddles tw[k1][b] = w_L^{b k1}, the spectral
-  // twiddles w^k (k < L), the CTA's kernel spectra g[c][k] (k <= L), then a
-  // transpose buffer per column.  The tables arrive by cp.async together with
-  // the columns' loads, so the kernel pays one memory latency, not one per step.
-  V* tws = reinterpret_cast<V*>(smem_raw);       // [E][S]
-  V* wks = tws + L;                              // [L]
-  float* gs = reinterpret_cast<float*>(wks + L); // [CPC][L + 1]
-  V* T = reinterpret_cast<V*>(gs + Sh::GS) + size_t(cl) * 2 * Sh::CB;   // two buffers a column
-  const V* w2 = a.w2_z;                          // w2[j] = e^{-2 pi i j / (2L)}, j < 2L
-  for (int i = int(threadIdx.x); i < L; i += 32 * kZWarps) {
-    const int k1 = i / S, bb = i % S;
-    cp_async8(tws + i, w2 + 2 * bb * k1);
-  }
-  for (int i = int(threadIdx.x); i < L / 2; i += 32 * kZWarps) cp_async16(wks + 2 * i, w2 + 2 * i);
-  {
-    const int nc = a.mc - col0 < CPC ? a.mc - col0 : CPC;
-    const float* g0 = a.gz + size_t(col0) * (L + 1);
-    for (int i = int(threadIdx.x); i < nc * (L + 1); i += 32 * kZWarps) cp_async4(gs + i, g0 + i);
-  }
-  cp_async_commit();
-
-  // 1. the packed column z(m) = x(2m) + i x(2m+1), m = b + S a < L/2, summed
-  //    over the groups of partial projections
-  V v[E];
+  const T* zp = a.zp + size_t(valid ? col : 0) * kModeZPar;
+  T par[kModeZPar];
 #pragma unroll
-  for (int i = 0; i < E; ++i) v[i] = make_float2(0.f, 0.f);
+  for (int i = 0; i < kModeZPar / EV; ++i) *reinterpret_cast<V*>(par + EV * i) = __ldg(reinterpret_cast<const V*>(zp) + i);
+  const T beta = par[0], gamma = par[1], p = sizeof(T) == 4 ? par[2] : par[3];
+  const T* w = par + 4;                           // w[i] = q^{kV 2^i}
+
+  // the column's values, summed over the groups of partial projections
+  T x[kV];
+#pragma unroll
+  for (int j = 0; j < kV; ++j) x[j] = T(0);
   if (valid) {
-#pragma unroll 4
+#pragma unroll 8
     for (int s = 0; s < groups; ++s) {
-      const V* src = reinterpret_cast<const V*>(a.part + (size_t(s) * a.mc + col) * L) + b;
+      const V* src = reinterpret_cast<const V*>(a.part + (size_t(s) * a.mc + col) * NZ + t * kV);
+      T g[kV];
 #pragma unroll
-      for (int i = 0; i < E / 2; ++i) {
-        const V z = __ldg(src + S * i);
-        v[i].x += z.x;
-        v[i].y += z.y;
-      }
+      for (int i = 0; i < kV / EV; ++i) *reinterpret_cast<V*>(g + EV * i) = __ldg(src + i);
+#pragma unroll
+      for (int j = 0; j < kV; ++j) x[j] += g[j];
     }
   }
-  cp_async_wait<0>();
-  __syncthreads();
-
-  // 2. forward transform
-  dft_reg<E, false>(v);                          // over a; inputs a >= E/2 are zero
+  // totals of the thread's values, then of all threads up to this one
+  T sf = x[0], sb = x[kV - 1];
 #pragma unroll
-  for (int k1 = 1; k1 < E; ++k1) v[k1] = cmul(v[k1], tws[k1 * S + b]);     // w_L^{b k1}
-#pragma unroll
-  for (int k1 = 0; k1 < E; ++k1) T[k1 * (S + 1) + b] = v[k1];
-  __syncwarp();
-#pragma unroll
-  for (int i = 0; i < E / S; ++i) {
-    V* u = v + i * S;
-#pragma unroll
-    for (int bb = 0; bb < S; ++bb) u[bb] = T[(b + S * i) * (S + 1) + bb];
-    dft_reg<S, false>(u);                        // over b: X(k1 + E k2), k1 = b + S i
+  for (int j = 1; j < kV; ++j) {
+    sf = zstep(sf, x[j], p);
+    sb = zstep(sb, x[kV - 1 - j], p);
   }
-  __syncwarp();
 #pragma unroll
-  for (int i = 0; i < E / S; ++i)
-#pragma unroll
-    for (int k2 = 0; k2 < S; ++k2) T[b + S * i + E * k2] = v[i * S + k2];
-  __syncwarp();
-
-  // 3. real spectrum, kernel product, packed inverse input Z'(k) into the
-  //    column's second buffer, then back to registers in the layout of the
-  //    inverse.  Each pair (k, L-k), k = b + S i < L/2, is formed once:
-  //    with s = Y(k) + conj Y(L-k) and t = conj(w^k) (Y(k) - conj Y(L-k)),
-  //    Z'(k) = s + i t and Z'(L-k) = conj(s) + i conj(t); lane b = 0 also
-  //    takes the self-paired k = L/2.  (A rolled loop: the code stays small
-  //    enough for the instruction cache.)
-  const float* g = gs + cl * (L + 1);
-  V* U = T + Sh::CB;
-  auto pair = [&](int k, bool both) {
-    const V zk = T[k], zm = T[(L - k) & (L - 1)];
-    const V wk = wks[k];                         // w^k
-    const V wm = make_float2(-wk.x, wk.y);       // w^{L-k} = -conj(w^k)
-    const float gk = valid ? g[k] : 0.f, gm = valid ? g[L - k] : 0.f;
-    auto unpack = [](V x, V xm, V w) {           // (x + conj xm - i w (x - conj xm)) / 2
-      const V c = cconj(xm);
-      const V su = cadd(x, c), df = csub(x, c);
-      const V wd = cmul(w, df);
-      return make_float2(0.5f * (su.x + wd.y), 0.5f * (su.y - wd.x));
-    };
-    const V yk = cscale(unpack(zk, zm, wk), gk);
-    const V ym = cscale(unpack(zm, zk, wm), gm);
-    const V c = cconj(ym);
-    const V sp = cadd(yk, c), d = csub(yk, c);
-    const V t = cmulc<true>(d, wk);
-    U[k] = make_float2(sp.x - t.y, sp.y + t.x);
-    if (both) U[L - k] = make_float2(sp.x + t.y, t.x - sp.y);
-  };
-#pragma unroll 2
-  for (int i = 0; i < E / 2; ++i) {
-    const int k = b + S * i;
-    pair(k, k != 0);
+  for (int i = 0; (1 << i) < SEG; ++i) {
+    const int d = 1 << i;
+    const T uf = __shfl_up_sync(0xffffffffu, sf, d, SEG), ub = __shfl_down_sync(0xffffffffu, sb, d, SEG);
+    if (ls >= d) sf = fma(w[i], uf, sf);
+    if (ls + d < SEG) sb = fma(w[i], ub, sb);
   }
-  if (b == 0) pair(L / 2, false);
-  __syncwarp();
+  T F = __shfl_up_sync(0xffffffffu, sf, 1, SEG), B = __shfl_down_sync(0xffffffffu, sb, 1, SEG);
+  if (ls == 0) F = T(0);
+  if (ls == SEG - 1) B = T(0);
+  if constexpr (NW > 1) {                         // the other warps of the column
+    const int warp = int(threadIdx.x) / 32, w0 = warp - wq;
+    if (ls == SEG - 1) tot[0][warp] = sf;
+    if (ls == 0) tot[1][warp] = sb;
+    __syncthreads();
+    T cf = T(0), cb = T(0);
 #pragma unroll
-  for (int i = 0; i < E; ++i) v[i] = U[b + S * i];
-
-  // 4. inverse transform; the outputs m = k1 + E k2 < L/2 (k2 < S/2) are psi
-  dft_reg<E, true>(v);
-#pragma unroll
-  for (int k1 = 1; k1 < E; ++k1) v[k1] = cmulc<true>(v[k1], tws[k1 * S + b]);
-#pragma unroll
-  for (int k1 = 0; k1 < E; ++k1) T[k1 * (S + 1) + b] = v[k1];
-  __syncwarp();
-  V* dst = reinterpret_cast<V*>(a.psi + size_t(valid ? col : 0) * L);
-#pragma unroll
-  for (int i = 0; i < E / S; ++i) {
-    V* u = v + i * S;
-#pragma unroll
-    for (int bb = 0; bb < S; ++bb) u[bb] = T[(b + S * i) * (S + 1) + bb];
-    dft_reg<S, true>(u);
-    if (valid) {
-#pragma unroll
-      for (int k2 = 0; k2 < S / 2; ++k2) dst[b + S * i + E * k2] = u[k2];
+    for (int u = 0; u < NW - 1; ++u) {
+      if (u < wq) cf = fma(w[5], cf, tot[0][w0 + u]);
+      if (NW - 1 - u > wq) cb = fma(w[5], cb, tot[1][w0 + NW - 1 - u]);
     }
+    T pf = T(1), pb = T(1);                       // q^{kV ls}, q^{kV (31 - ls)}
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      if (ls >> i & 1) pf *= w[i];
+      else pb *= w[i];
+    }
+    F = fma(pf, cf, F);
+    B = fma(pb, cb, B);
+  }
+  T f[kV];
+#pragma unroll
+  for (int j = 0; j < kV; ++j) {
+    f[j] = F;
+    F = zstep(F, x[j], p);
+  }
+#pragma unroll
+  for (int j = kV - 1; j >= 0; --j) {
+    f[j] = fma(gamma, f[j] + B, beta * x[j]);
+    B = zstep(B, x[j], p);
+  }
+  if (valid) {
+    V* dst = reinterpret_cast<V*>(a.psi + size_t(col) * NZ + t * kV);
+#pragma unroll
+    for (int i = 0; i < kV / EV; ++i) dst[i] = *reinterpret_cast<const V*>(f + EV * i);
   }
 }
 
-template <int L>
-__global__ void __launch_bounds__(32 * kZWarps) mode_z_warp_kernel(ModeArgs<float> a, int groups) {
-  z_warp<L>(a, groups, int(blockIdx.x));
+template <typename T, int NZ>
+__global__ void __launch_bounds__(kZThreads) mode_z_kernel(ModeArgs<T> a, int groups) {
+  z_scan<T, NZ>(a, groups, int(blockIdx.x));
 }
 
 // a group of solves of one shape: solve s takes the CTAs s * cps .. (s + 1) * cps - 1
-template <int L>
-__global__ void __launch_bounds__(32 * kZWarps) mode_z_warp_group_kernel(const __grid_constant__ ModeGroup g,
-                                                                          int groups, int cps) {
-  const int s = int(blockIdx.x) / cps;
-  const ModeArgs<float> a = g.args[s];
-  z_warp<L>(a, groups, int(blockIdx.x) % cps);
+template <int NZ>
+__global__ void __launch_bounds__(kZThreads) mode_z_group_kernel(const __grid_constant__ ModeGroup g, int groups,
+                                                                 int cps) {
+  const ModeArgs<float> a = g.args[int(blockIdx.x) / cps];
+  z_scan<float, NZ>(a, groups, int(blockIdx.x) % cps);
 }
 
-template <int L>
-cudaError_t launch_zw(const ModeArgs<float>& a, int groups, const ModeGroup* g, cudaStream_t st) {
-  using Sh = ZWarpShape<L>;
-  const int per = kZWarps * Sh::CPW;             // columns per CTA
-  const int cps = (a.mc + per - 1) / per;        // CTAs per solve
-  void (*kern)(ModeArgs<float>, int) = mode_z_warp_kernel<L>;
-  void (*gkern)(const ModeGroup, int, int) = mode_z_warp_group_kernel<L>;
-  if (Sh::SMEM > 48 * 1024) {
-    const cudaError_t e = g ? cudaFuncSetAttribute(gkern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(Sh::SMEM))
-                            : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(Sh::SMEM));
-    if (e != cudaSuccess) return e;
+template <typename T, int NZ>
+cudaError_t launch_z_nz(const ModeArgs<T>& a, int groups, const ModeGroup* g, cudaStream_t st) {
+  constexpr int per = kZThreads * kV / NZ;        // columns per CTA
+  const int cps = (a.mc + per - 1) / per;         // CTAs per solve
+  if constexpr (sizeof(T) == 4) {
+    if (g) {
+      mode_z_group_kernel<NZ><<<g->n * cps, kZThreads, 0, st>>>(*g, groups, cps);
+      return cudaGetLastError();
+    }
   }
-  if (g) gkern<<<g->n * cps, 32 * kZWarps, Sh::SMEM, st>>>(*g, groups, cps);
-  else kern<<<cps, 32 * kZWarps, Sh::SMEM, st>>>(a, groups);
+  mode_z_kernel<T, NZ><<<cps, kZThreads, 0, st>>>(a, groups);
   return cudaGetLastError();
 }
 
-cudaError_t launch_zw_any(const ModeArgs<float>& a, int groups, const ModeGroup* g, cudaStream_t st) {
+template <typename T>
+cudaError_t launch_z_any(const ModeArgs<T>& a, int groups, const ModeGroup* g, cudaStream_t st) {
   switch (a.nz) {
-    case 32: return launch_zw<32>(a, groups, g, st);
-    case 64: return launch_zw<64>(a, groups, g, st);
-    case 128: return launch_zw<128>(a, groups, g, st);
-    case 256: return launch_zw<256>(a, groups, g, st);
-    case 512: return launch_zw<512>(a, groups, g, st);
-    case 1024: return launch_zw<1024>(a, groups, g, st);
+    case 32: return launch_z_nz<T, 32>(a, groups, g, st);
+    case 64: return launch_z_nz<T, 64>(a, groups, g, st);
+    case 128: return launch_z_nz<T, 128>(a, groups, g, st);
+    case 256: return launch_z_nz<T, 256>(a, groups, g, st);
+    case 512: return launch_z_nz<T, 512>(a, groups, g, st);
+    case 1024: return launch_z_nz<T, 1024>(a, groups, g, st);
     default: return cudaErrorInvalidValue;
   }
 }
 
 }  // namespace
 
-cudaError_t launch_mode_z_warp(const ModeArgs<float>& a, int groups, cudaStream_t st) {
-  return launch_zw_any(a, groups, nullptr, st);
+template <typename T>
+cudaError_t launch_mode_z(const ModeArgs<T>& a, int groups, cudaStream_t st) {
+  return launch_z_any<T>(a, groups, nullptr, st);
 }
+template cudaError_t launch_mode_z<float>(const ModeArgs<float>&, int, cudaStream_t);
+template cudaError_t launch_mode_z<double>(const ModeArgs<double>&, int, cudaStream_t);
 
-cudaError_t launch_mode_z_warp_group(const ModeArgs<float>& a, int groups, const ModeGroup& g, cudaStream_t st) {
+cudaError_t launch_mode_z_group(const ModeArgs<float>& a, int groups, const ModeGroup& g, cudaStream_t st) {
   if (g.n < 1 || g.n > kMaxModeGroup) return cudaErrorInvalidValue;
-  return launch_zw_any(a, groups, &g, st);
+  return launch_z_any<float>(a, groups, &g, st);
 }
 
 }  // namespace pp
