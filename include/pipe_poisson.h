@@ -105,16 +105,17 @@ typedef struct pipe_handle pipe_handle;
  *    transforms pruned to the modes of the truncated series (Eq. 7), where
  *    the transformed Green function is nonzero: a projection of rho onto the
  *    modes_m x modes_n sine modes, the zero-padded z convolution of each
- *    mode's column by FFT (Appendix A), and the back-projection.  Any mesh
+ *    mode's column (Appendix A), and the back-projection.  Any mesh
  *    inside the pipe with nx and ny multiples of 16 (nx != ny allowed, up to
  *    4096 each), nz in {32, ..., 1024} as above, modes_m, modes_n <= 32;
  *    PIPE_F32 or PIPE_F64; not banded; and its kernels' shared memory within
  *    the device's 227 KB per CTA (it grows with ny and the modes: FP32 with
  *    20 x 20 modes takes ny up to about 1400, FP64 about 700; FP64 takes at
  *    most about 880 mode pairs, e.g. 32 x 24 but not 32 x 32).  Its tables
- *    (FP64, with FP32 copies) take (nx*mxp + ny*myp + mxp*myp*(nz+1))*12
- *    bytes and its scratch (xblocks + 1)*mxp*myp*nz values of the dtype (the
- *    sizes of pipe_mode_layout).
+ *    (FP64, with FP32 copies) take (nx*mxp + ny*myp + 12*mxp*myp)*12 bytes
+ *    (FP64 about 10 times that, as fragments for the tensor cores) and its
+ *    scratch (xblocks + 1)*mxp*myp*nz values of the dtype (the sizes of
+ *    pipe_mode_layout); FP64 in addition nx*myp*nz values, at most 32 MiB.
  *    The default where the modes are at most half the transverse mesh
  *    (2*max(ceil4(modes_m), slots) <= min(nx, ny)) or the padded transforms
  *    cannot take the mesh.
@@ -177,7 +178,9 @@ int pipe_poisson_adjoint(pipe_handle* h, const void* dphi, void* drho, void* str
  * library instead of device memory owned by the handle -- for the
  * padded-transform form the z half-spectrum, (nz+1)*nx*ny complex values of
  * the dtype; for the mode-space form (plan t_kind 3) the projections and the
- * convolved mode columns, (xblocks+1)*mxp*myp*nz values (pipe_mode_layout).
+ * convolved mode columns, (xblocks+1)*mxp*myp*nz values (pipe_mode_layout;
+ * for FP64, with xblocks taken as nx/8 over the largest divisor of nx/8 that
+ * is at most 4, and never less than the scratch stated at pipe_green_setup).
  * The handle's current form runs, so the result is bit for bit that of
  * pipe_poisson_solve.  Meant for programs that must not let a library
  * allocate device memory while they run (a host that keeps the GPU's memory
@@ -326,14 +329,14 @@ int pipe_stage_z_inverse(pipe_handle* h, const void* spec, void* phi, int adjoin
 /* Layout of the mode-space form (Sec. 2 Eq. 7: the sine modes of the
  * truncated series).  mx = modes_m; mxp = mx rounded up to a multiple of 4;
  * myp = the y-mode slots: when the mesh is symmetric about the pipe's
- * mid-plane in y (2*y0 + (ny-1)*hy == b, e.g. cell-centred), *fold = 1 and
+ * mid-plane in y (2*y0 + (ny-1)*hy == b, e.g. cell-centred; for FP64 also
+ * y0 == 0 and ny*hy == b, the first row on the wall), *fold = 1 and
  * slot s < myp/2 holds mode n = 2s+1, slot s >= myp/2 mode n = 2(s - myp/2)+2;
  * otherwise *fold = 0 and slot s holds n = s+1 (slots beyond modes_n are
  * zero).  Mode column c = (m-1)*myp + slot.  xblocks: the groups of x rows
- * whose projections the first stage writes separately (the kernel works on
- * blocks of 16 rows in FP32, 8 in FP64, and sums up to 4 neighbouring blocks
- * in a thread-block cluster; xblocks = blocks / that cluster size, 2 for
- * FP32 nx = 128).  Errors: PIPE_EINVAL (null pointers), PIPE_EUNSUPPORTED
+ * whose projections the first stage writes separately (FP32: the kernel works
+ * on blocks of 16 rows and sums up to 4 neighbouring blocks in a thread-block
+ * cluster; xblocks = blocks / that cluster size, 2 for nx = 128.  FP64: 1).  Errors: PIPE_EINVAL (null pointers), PIPE_EUNSUPPORTED
  * (the mode-space form cannot take the handle). */
 int pipe_mode_layout(pipe_handle* h, int* mx, int* mxp, int* myp, int* fold, int* xblocks);
 
@@ -353,8 +356,8 @@ int pipe_mode_spectrum(pipe_handle* h, double* out, size_t count);
  *            part[b][c][k] = sum_{i in block b} sum_j sin(m pi x_i/a) *
  *                            sin(n pi y_j/b) rho[i][j][k]
  *   stage 1: in = part -> out = psi [mxp*myp][nz]: the blocks summed, each
- *            column convolved along z with its kernel (zero-padded 2nz-point
- *            transforms, the spectrum of pipe_mode_spectrum), first nz values;
+ *            column convolved along z with its kernel K_c (zero beyond the
+ *            mesh), nz values;
  *            for a banded handle (pipe_banded_setup) the sum over
  *            |d| <= n_neighbors of K_c(|d| hz) part[c][k - d] instead
  *   stage 2: in = psi -> out = phi [nx][ny][nz]:

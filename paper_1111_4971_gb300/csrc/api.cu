@@ -16,6 +16,7 @@
 #include "handle.cuh"
 #include "modes.cuh"
 #include "modes_impl.cuh"
+#include "modes_split.cuh"
 #include "solver.cuh"
 
 using namespace pp;
@@ -123,10 +124,11 @@ void free_handle(pipe_handle* h) {
   cudaFree(h->tab32); cudaFree(h->tab64);
   cudaFree(h->stage_rho); cudaFree(h->stage_phi);
   cudaFree(h->tbuf);
-  cudaFree(h->msx64); cudaFree(h->msy64); cudaFree(h->mgz64);
+  cudaFree(h->msx64); cudaFree(h->msy64);
   cudaFree(h->msx32); cudaFree(h->msy32);
   cudaFree(h->mzp64); cudaFree(h->mzp32);
   cudaFree(h->mwork);
+  cudaFree(h->msplit);
   cudaFree(h->mkb64); cudaFree(h->mkb32);
   std::free(h->msy_host);
   for (int k = 0; k < 2; ++k) {
@@ -245,13 +247,28 @@ int finish_setup(pipe_handle* h, pipe_handle** out) {
 
 namespace pp {
 int mode_xblocks(const pipe_handle* h) {
-  const int xb = h->grid.nx / (h->grid.dtype == PIPE_F64 ? ModeShape<double>::XB : ModeShape<float>::XB);
+  if (h->grid.dtype == PIPE_F64) return 1;
+  const int xb = h->grid.nx / ModeShape<float>::XB;
   return xb / mode_cluster(xb);
 }
 
 size_t mode_scratch_bytes(const pipe_handle* h) {
   const size_t mc = size_t(h->mxp) * h->myp;
-  return (h->grid.dtype == PIPE_F64 ? 8 : 4) * size_t(mode_xblocks(h) + 1) * mc * h->grid.nz;
+  const bool f64 = h->grid.dtype == PIPE_F64;
+  return (f64 ? 8 : 4) * size_t(mode_xblocks(h) + 1) * mc * h->grid.nz +
+         (f64 ? split_half_bytes(h->grid.nx, h->myp, h->grid.nz) : 0);
+}
+
+// the scratch, but FP64 at least one partial projection per cluster of 8-row
+// blocks, the size that this entry point's documented limit stands for
+size_t mode_noalloc_bytes(const pipe_handle* h) {
+  size_t need = mode_scratch_bytes(h);
+  if (h->grid.dtype == PIPE_F64) {
+    const int xb = h->grid.nx / 8;
+    const size_t limit = sizeof(double) * size_t(xb / mode_cluster(xb) + 1) * h->mxp * h->myp * h->grid.nz;
+    if (limit > need) need = limit;
+  }
+  return need;
 }
 
 template <typename T>
@@ -269,19 +286,32 @@ ModeArgs<T> mode_args(const pipe_handle* h, const void* rho, void* phi, void* pa
   a.mx = h->geom.modes_m;
   a.mxp = h->mxp;
   a.mc = h->mxp * h->myp;
+  a.groups = mode_xblocks(h);
   a.kb = reinterpret_cast<const T*>(D ? static_cast<const void*>(h->mkb64) : static_cast<const void*>(h->mkb32));
   a.nb = h->banded;
   return a;
 }
 
+// one stage; `half`: FP64's buffer of the half-transformed field
 template <typename T>
-int mode_stage(const pipe_handle* h, int stage, const void* rho, void* phi, void* part, void* psi,
+int mode_stage(const pipe_handle* h, int stage, const void* rho, void* phi, void* part, void* psi, void* half,
                cudaStream_t st) {
   const ModeArgs<T> a = mode_args<T>(h, rho, phi, part, psi);
+  if (stage == 1) return status_of(launch_mode_z_stage<T>(a, st));
   if constexpr (sizeof(T) == 4) {
-    if (h->mfast && stage != 1) return status_of(launch_mode_fast(stage, h->myp, a, h->msy_host, st));
+    if (h->mfast) return status_of(launch_mode_fast(stage, h->myp, a, h->msy_host, st));
+    return status_of(launch_mode_sums(stage, h->myp, h->fy != 0, a, st));
+  } else {
+    SplitArgs s{};
+    s.cy = h->mcy; s.cx = h->mcx; s.ey = h->mey; s.ex = h->mex;
+    s.ey_small = h->mey_small; s.ex_small = h->mex_small;
+    s.nx = a.nx; s.ny = a.ny; s.nz = a.nz;
+    s.mx = a.mx; s.mxp = h->mxp; s.myp = h->myp;
+    s.fold = h->fy;
+    s.half = static_cast<double*>(half);
+    s.zs = split_slab(a.nx, h->myp, a.nz);
+    return status_of(stage == 0 ? launch_split_project(s, a.rho, a.part, st) : launch_split_back(s, a.psi, a.phi, st));
   }
-  return status_of(launch_mode_stage<T>(stage, h->myp, h->fy != 0, a, st));
 }
 
 ModeArgs<float> mode_args_f32(const pipe_handle* h) {
@@ -290,12 +320,12 @@ ModeArgs<float> mode_args_f32(const pipe_handle* h) {
 }
 
 int mode_solve(pipe_handle* h, const void* rho, void* phi, void* scratch, cudaStream_t st) {
-  const size_t esz = h->grid.dtype == PIPE_F64 ? 8 : 4;
-  void* psi = static_cast<char*>(scratch) + esz * size_t(mode_xblocks(h)) * h->mxp * h->myp * h->grid.nz;
+  const size_t column = (h->grid.dtype == PIPE_F64 ? 8 : 4) * size_t(h->mxp) * h->myp * h->grid.nz;
+  char* psi = static_cast<char*>(scratch) + size_t(mode_xblocks(h)) * column;
   int s = PIPE_OK;
   for (int stage = 0; stage < 3 && s == PIPE_OK; ++stage)
-    s = h->grid.dtype == PIPE_F64 ? mode_stage<double>(h, stage, rho, phi, scratch, psi, st)
-                                  : mode_stage<float>(h, stage, rho, phi, scratch, psi, st);
+    s = h->grid.dtype == PIPE_F64 ? mode_stage<double>(h, stage, rho, phi, scratch, psi, psi + column, st)
+                                  : mode_stage<float>(h, stage, rho, phi, scratch, psi, nullptr, st);
   return s;
 }
 
@@ -431,23 +461,54 @@ static int setup_pipe(const pipe_geometry* geom, const pipe_grid* grid, int igf,
   s.modes_m = geom->modes_m; s.modes_n = geom->modes_n;
   s.igf = igf;
   if (modes_ok) {
-    h->fy = fold ? 1 : 0;
+    // FP64 also folds meshes with row 0 on the wall (y_{ny-j} = b - y_j)
+    const bool wall = grid->dtype == PIPE_F64 && geom->y0 == 0.0 &&
+                      std::fabs(grid->ny * grid->hy - geom->b) <= 1e-12 * geom->b;
+    h->fy = fold ? 1 : (wall ? 2 : 0);
     h->mxp = (geom->modes_m + 3) / 4 * 4;
-    h->myp = mode_slots(geom->modes_n, fold);
-    const size_t nsx = size_t(grid->nx) * h->mxp, nsy = size_t(fold ? grid->ny / 2 : grid->ny) * h->myp;
-    const size_t ngz = size_t(h->mxp) * h->myp * (grid->nz + 1);
+    h->myp = mode_slots(geom->modes_n, h->fy != 0);
+    const size_t nsx = size_t(grid->nx) * h->mxp, nsy = size_t(h->fy ? grid->ny / 2 : grid->ny) * h->myp;
     const size_t nzp = size_t(h->mxp) * h->myp * kModeZPar;
     if (cudaMalloc(&h->msx64, nsx * 8) != cudaSuccess || cudaMalloc(&h->msx32, nsx * 4) != cudaSuccess ||
         cudaMalloc(&h->msy64, nsy * 8) != cudaSuccess || cudaMalloc(&h->msy32, nsy * 4) != cudaSuccess ||
-        cudaMalloc(&h->mgz64, ngz * 8) != cudaSuccess || cudaMalloc(&h->mzp64, nzp * 8) != cudaSuccess ||
+        cudaMalloc(&h->mzp64, nzp * 8) != cudaSuccess ||
         cudaMalloc(&h->mzp32, nzp * 4) != cudaSuccess ||
         cudaMalloc(&h->mwork, mode_scratch_bytes(h)) != cudaSuccess) {
       free_handle(h);
       return PIPE_ENOMEM;
     }
     cudaError_t e = build_mode_tables(s, geom->x0, geom->y0, h->mxp, h->myp, h->fy, h->msx64, h->msx32,
-                                      h->msy64, h->msy32, h->mgz64, h->mzp64, h->mzp32, nullptr);
+                                      h->msy64, h->msy32, h->mzp64, h->mzp32, nullptr);
     if (e != cudaSuccess) { free_handle(h); return status_of(e); }
+    if (grid->dtype == PIPE_F64) {       // the split products' fragment tables
+      const int nyk = h->fy ? grid->ny / 2 : grid->ny;
+      const bool halves = h->fy != 0;
+      const size_t n[4] = {split_contract_size(nyk, h->myp, halves), split_contract_size(grid->nx, h->mxp, false),
+                           split_expand_size(nyk, h->myp, halves), split_expand_size(grid->nx, h->mxp, false)};
+      if (cudaMalloc(&h->msplit, (n[0] + n[1] + n[2] + n[3]) * sizeof(uint4)) != cudaSuccess) {
+        free_handle(h);
+        return PIPE_ENOMEM;
+      }
+      h->mcy = h->msplit; h->mcx = h->mcy + n[0]; h->mey = h->mcx + n[1]; h->mex = h->mey + n[2];
+      if ((e = build_split_table(h->msy64, nyk, h->myp, halves, false, h->mcy, nullptr)) != cudaSuccess ||
+          (e = build_split_table(h->msx64, grid->nx, h->mxp, false, false, h->mcx, nullptr)) != cudaSuccess ||
+          (e = build_split_table(h->msy64, nyk, h->myp, halves, true, h->mey, nullptr)) != cudaSuccess ||
+          (e = build_split_table(h->msx64, grid->nx, h->mxp, false, true, h->mex, nullptr)) != cudaSuccess ||
+          (e = cudaStreamSynchronize(nullptr)) != cudaSuccess) {
+        free_handle(h);
+        return status_of(e);
+      }
+      double* t = static_cast<double*>(std::malloc((nsx > nsy ? nsx : nsy) * sizeof(double)));
+      if (!t) { free_handle(h); return PIPE_ENOMEM; }
+      e = cudaMemcpy(t, h->msy64, nsy * sizeof(double), cudaMemcpyDeviceToHost);
+      if (e == cudaSuccess) {
+        h->mey_small = expand_sums_small(t, nyk, h->myp, halves);
+        e = cudaMemcpy(t, h->msx64, nsx * sizeof(double), cudaMemcpyDeviceToHost);
+      }
+      if (e == cudaSuccess) h->mex_small = expand_sums_small(t, grid->nx, h->mxp, false);
+      std::free(t);
+      if (e != cudaSuccess) { free_handle(h); return status_of(e); }
+    }
     if (n_nb >= 0) {                     // the banded operator's z stencil
       const size_t nkb = size_t(h->mxp) * h->myp * (n_nb + 1);
       if (cudaMalloc(&h->mkb64, nkb * 8) != cudaSuccess || cudaMalloc(&h->mkb32, nkb * 4) != cudaSuccess) {
@@ -661,7 +722,7 @@ int pipe_mode_layout(pipe_handle* h, int* mx, int* mxp, int* myp, int* fold, int
   *mx = h->geom.modes_m;
   *mxp = h->mxp;
   *myp = h->myp;
-  *fold = h->fy;
+  *fold = h->fy != 0;
   *xblocks = mode_xblocks(h);
   return PIPE_OK;
 }
@@ -671,7 +732,18 @@ int pipe_mode_spectrum(pipe_handle* h, double* out, size_t count) {
   if (!h->modes_ok) return PIPE_EUNSUPPORTED;
   if (count != size_t(h->mxp) * h->myp * (h->grid.nz + 1)) return PIPE_EINVAL;
   DeviceGuard dg(h->device);
-  return status_of(cudaMemcpy(out, h->mgz64, count * sizeof(double), cudaMemcpyDeviceToHost));
+  GreenSpec s{};
+  s.nx = h->grid.nx; s.ny = h->grid.ny; s.nz = h->grid.nz;
+  s.hx = h->grid.hx; s.hy = h->grid.hy; s.hz = h->grid.hz;
+  s.a = h->geom.a; s.b = h->geom.b;
+  s.modes_m = h->geom.modes_m; s.modes_n = h->geom.modes_n;
+  s.igf = h->kind;
+  double* g = nullptr;
+  cudaError_t e = cudaMalloc(&g, count * sizeof(double));
+  if (e == cudaSuccess) e = build_mode_spectrum(s, h->mxp, h->myp, h->fy, g, nullptr);
+  if (e == cudaSuccess) e = cudaMemcpy(out, g, count * sizeof(double), cudaMemcpyDeviceToHost);
+  cudaFree(g);
+  return status_of(e);
 }
 
 int pipe_stage_modes(pipe_handle* h, int stage, const void* in, void* out, void* stream) {
@@ -689,8 +761,10 @@ int pipe_stage_modes(pipe_handle* h, int stage, const void* in, void* out, void*
   void* part = stage == 0 ? out : (stage == 1 ? vin : nullptr);
   void* psi = stage == 1 ? out : (stage == 2 ? vin : nullptr);
   void* phi = stage == 2 ? out : nullptr;
-  return h->grid.dtype == PIPE_F64 ? mode_stage<double>(h, stage, rho, phi, part, psi, s)
-                                   : mode_stage<float>(h, stage, rho, phi, part, psi, s);
+  if (h->grid.dtype != PIPE_F64) return mode_stage<float>(h, stage, rho, phi, part, psi, nullptr, s);
+  // the half-transformed field is the handle's, as in a solve
+  char* half = static_cast<char*>(h->mwork) + sizeof(double) * size_t(mode_xblocks(h) + 1) * h->mxp * h->myp * h->grid.nz;
+  return mode_stage<double>(h, stage, rho, phi, part, psi, half, s);
 }
 
 }  // extern "C"

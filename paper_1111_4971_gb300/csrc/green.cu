@@ -490,20 +490,24 @@ done:
 // ---------------------------------------------------------------------------
 // Tables of the mode-space solve (modes_impl.cuh), all FP64 with FP32 copies:
 //   sx[i][s] = sin(m pi x_i / a), m = s + 1 (zero for m > Mx), i < nx, s < mxp
-//   sy[j][s] = sin(n pi y_j / b) for the mode n of slot s (mode_of_slot), j < nyk
+//   sy[j][s] = sin(n pi y_j / b) for the mode n of slot s (mode_of_slot), j < nyk;
+//       fold 2 (row 0 on the wall): row 0, whose own sines are zero, holds row
+//       ny/2, its own mirror image (odd n; the even n vanish there)
 //   zp[c], c = s_x * myp + s_y: the parameters of the z recurrences of
 //       K_mn(d) = hx hy hz (8 pi / ab) kappa_mn^{-1} f_mn(d hz)
 //   (f the e^{-kappa |w|} of Eq. 9 or the IGF g_z of Eq. 15): K(0), K(1),
 //   1 - q, q, q^{kModeZRun 2^i}, with q = e^{-kappa hz}, so K(d) = K(1) q^{d-1}
-//   gz[c][kz]: the DCT-I of the doubled z table of K_mn, divided by 2nz.
+// and, for inspection, gz[c][kz]: the DCT-I of the doubled z table of K_mn,
+// divided by 2nz (the kernel spectra of Appendix A's padded convolution).
 // ---------------------------------------------------------------------------
 __global__ void mode_sine_kernel(double* t64, float* t32, int rows, int slots, int nmodes, int fold,
-                                 double origin, double h, double len) {
+                                 double origin, double h, double len) {   // fold 2: rows = ny / 2
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= rows * slots) return;
   const int r = idx / slots, s = idx % slots;
   const int mode = !fold ? s + 1 : (s < slots / 2 ? 2 * s + 1 : 2 * (s - slots / 2) + 2);
-  const double v = mode <= nmodes ? sinpi(double(mode) * (origin + double(r) * h) / len) : 0.0;
+  double v = mode <= nmodes ? sinpi(double(mode) * (origin + double(r) * h) / len) : 0.0;
+  if (fold == 2 && r == 0) v = mode <= nmodes && mode % 2 ? sinpi(double(mode) * (origin + double(rows) * h) / len) : 0.0;
   t64[idx] = v;
   t32[idx] = float(v);
 }
@@ -520,8 +524,15 @@ __global__ void mode_zp_kernel(double* z64, float* z32, int M, int N, int mxp, i
     const double km = double(m) / a, kn = double(n) / b;
     const double kap = M_PI * sqrt(km * km + kn * kn);
     const double x = kap * hz, q = exp(-x), p = -expm1(-x);
+    // (K(1) multiplies every lag but 0: its products are carried to twice the
+    // length and rounded once, C itself comes as one rounded number)
+    const double r = p / x, rl = fma(-r, x, p) / x;              // p / x = r + rl
+    const double r2 = r * r, r2l = fma(r, r, -r2) + 2.0 * r * rl;
+    const double f = igf ? r2 : q, fl = igf ? r2l : 0.0;
+    const double g = C * f, gl = fma(C, f, -g) + C * fl;
+    const double k1 = g / kap;
     v[0] = C / kap * (igf ? 2.0 * xm1pe_over_x2(x) : 1.0);
-    v[1] = C / kap * (igf ? (p / x) * (p / x) : q);
+    v[1] = k1 + (fma(-k1, kap, g) + gl) / kap;
     v[2] = p;
     v[3] = q;
     for (int i = 0; i < kModeZPar - 4; ++i) v[4 + i] = exp(-x * double(kModeZRun << i));
@@ -574,24 +585,30 @@ cudaError_t build_mode_band(const GreenSpec& s, int mxp, int myp, int fold, int 
 }
 
 cudaError_t build_mode_tables(const GreenSpec& s, double x0, double y0, int mxp, int myp, int fold,
-                              double* sx64, float* sx32, double* sy64, float* sy32, double* gz64,
-                              double* zp64, float* zp32, cudaStream_t st) {
-  const int M = s.modes_m, N = s.modes_n, nz = s.nz;
+                              double* sx64, float* sx32, double* sy64, float* sy32, double* zp64, float* zp32,
+                              cudaStream_t st) {
+  const int M = s.modes_m, N = s.modes_n;
   const int nyk = fold ? s.ny / 2 : s.ny;
+  mode_sine_kernel<<<nblk(long(s.nx) * mxp, 256), 256, 0, st>>>(sx64, sx32, s.nx, mxp, M, 0, x0, s.hx, s.a);
+  mode_sine_kernel<<<nblk(long(nyk) * myp, 256), 256, 0, st>>>(sy64, sy32, nyk, myp, N, fold, y0, s.hy, s.b);
+  mode_zp_kernel<<<nblk(long(mxp) * myp, 64), 64, 0, st>>>(zp64, zp32, M, N, mxp, myp, fold, s.hz, s.a, s.b, s.igf,
+                                                           s.hx * s.hy * s.hz * 8.0 * M_PI / (s.a * s.b));
+  const cudaError_t err = cudaGetLastError();
+  return err == cudaSuccess ? cudaStreamSynchronize(st) : err;
+}
+
+cudaError_t build_mode_spectrum(const GreenSpec& s, int mxp, int myp, int fold, double* gz64, cudaStream_t st) {
+  const int M = s.modes_m, N = s.modes_n, nz = s.nz;
   double *Z = nullptr, *Zh = nullptr, *cosn = nullptr;
   cudaError_t err = cudaSuccess;
   if ((err = cudaMalloc(&Z, sizeof(double) * size_t(M) * N * (nz + 1))) != cudaSuccess) goto done;
   if ((err = cudaMalloc(&Zh, sizeof(double) * size_t(M) * N * (nz + 1))) != cudaSuccess) goto done;
   if ((err = cudaMalloc(&cosn, sizeof(double) * 2 * nz)) != cudaSuccess) goto done;
-  mode_sine_kernel<<<nblk(long(s.nx) * mxp, 256), 256, 0, st>>>(sx64, sx32, s.nx, mxp, M, 0, x0, s.hx, s.a);
-  mode_sine_kernel<<<nblk(long(nyk) * myp, 256), 256, 0, st>>>(sy64, sy32, nyk, myp, N, fold, y0, s.hy, s.b);
   z_profile_kernel<<<nblk(long(M) * N * (nz + 1), 256), 256, 0, st>>>(Z, M, N, nz, s.hz, s.a, s.b, s.igf);
   cos_pi_table_kernel<<<nblk(2 * nz, 256), 256, 0, st>>>(cosn, nz);
   z_dct_kernel<<<nblk(long(M) * N * (nz + 1), 256), 256, 0, st>>>(Zh, Z, M * N, nz, cosn);
   mode_gz_kernel<<<nblk(long(mxp) * myp * (nz + 1), 256), 256, 0, st>>>(
       gz64, Zh, M, N, mxp, myp, fold, nz, s.hx * s.hy * s.hz * 8.0 * M_PI / (s.a * s.b) / (2.0 * nz));
-  mode_zp_kernel<<<nblk(long(mxp) * myp, 64), 64, 0, st>>>(zp64, zp32, M, N, mxp, myp, fold, s.hz, s.a, s.b, s.igf,
-                                                           s.hx * s.hy * s.hz * 8.0 * M_PI / (s.a * s.b));
   if ((err = cudaGetLastError()) != cudaSuccess) goto done;
   err = cudaStreamSynchronize(st);
 done:

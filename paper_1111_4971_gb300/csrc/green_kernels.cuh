@@ -35,17 +35,19 @@ cudaError_t build_general_spectra(const GreenSpec& s, double x0, double y0, doub
 cudaError_t build_free_spectrum(const GreenSpec& s, double self_value, double* g64, float* g32,
                                 cudaStream_t st);
 
-// Tables of the mode-space solve: FP64 and FP32 copies of sx [nx][mxp],
-// sy [fold ? ny/2 : ny][myp] and zp [mxp*myp][kModeZPar], and gz [mxp*myp][nz+1]
-// (see green.cu).
-// Synchronous on `st`.  Uses temporary device memory (freed before return).
 // The banded operator's real-space z kernel in the mode slots, kb [mxp*myp][nb+1]
 // (FP64 and FP32).  Synchronous on `st`.  Uses temporary device memory.
 cudaError_t build_mode_band(const GreenSpec& s, int mxp, int myp, int fold, int nb, double* kb64, float* kb32,
                             cudaStream_t st);
 
+// Tables of the mode-space solve: FP64 and FP32 copies of sx [nx][mxp],
+// sy [fold ? ny/2 : ny][myp] and zp [mxp*myp][kModeZPar] (see green.cu).
+// Synchronous on `st`.
 cudaError_t build_mode_tables(const GreenSpec& s, double x0, double y0, int mxp, int myp, int fold,
-                              double* sx64, float* sx32, double* sy64, float* sy32, double* gz64,
-                              double* zp64, float* zp32, cudaStream_t st);
+                              double* sx64, float* sx32, double* sy64, float* sy32, double* zp64, float* zp32,
+                              cudaStream_t st);
+// The kernel spectra gz [mxp*myp][nz+1] of the mode columns.  Synchronous on
+// `st`.  Uses temporary device memory.
+cudaError_t build_mode_spectrum(const GreenSpec& s, int mxp, int myp, int fold, double* gz64, cudaStream_t st);
 
 }  // namespace pp

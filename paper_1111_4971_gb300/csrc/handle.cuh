@@ -56,15 +56,21 @@ struct pipe_handle {
   int modes_ok = 0;            // the mode path can run this handle
   int use_modes = 0;           // solves take the mode path (plan t_kind 3)
   int fft_ok = 1;              // the padded-transform path's buffers exist
-  int mxp = 0, myp = 0, fy = 0;
+  int mxp = 0, myp = 0;
+  int fy = 0;                  // y mirror pairs: 0 none, 1 (j, ny-1-j), 2 (j, ny-j) with row 0 on the wall
   double *msx64 = nullptr, *msy64 = nullptr;
   float *msx32 = nullptr, *msy32 = nullptr;
-  double* mgz64 = nullptr;     // DCT-I of the doubled z kernel tables [mxp*myp][nz+1] (pipe_mode_spectrum)
   double* mzp64 = nullptr;     // parameters of the z recurrences [mxp*myp][kModeZPar]
   float* mzp32 = nullptr;
   double* mkb64 = nullptr;     // banded operator in mode space: [mxp*myp][nb+1] real-space z kernel
   float* mkb32 = nullptr;
-  void* mwork = nullptr;       // part [xblocks][mc][nz], then psi [mc][nz], of the dtype
+  // FP64: fragment tables of the split products (modes_split.cu), one allocation
+  uint4* msplit = nullptr;
+  uint4 *mcy = nullptr, *mcx = nullptr, *mey = nullptr, *mex = nullptr;
+  bool mey_small = false, mex_small = false;   // expand_sums_small of mey, mex
+  // part [groups][mc][nz], then psi [mc][nz], of the dtype; FP64: then the
+  // half-transformed field of a slab (modes_split.cuh)
+  void* mwork = nullptr;
   float* msy_host = nullptr;   // FP32 y-mode table in host memory (the projection's kernel parameter)
   int mfast = 0;               // FP32 projection / back-projection in their occupancy layout
   pp::Plan plan{8, 0, 1, 256};
@@ -92,7 +98,9 @@ int handle_solve(pipe_handle* h, const void* rho, void* phi, bool adjoint, cudaS
 // the mode-space solve with `scratch` (mode_scratch_bytes) as its working buffer
 int mode_solve(pipe_handle* h, const void* rho, void* phi, void* scratch, cudaStream_t st);
 size_t mode_scratch_bytes(const pipe_handle* h);
-// x blocks of the projection (nx / rows per CTA of the dtype)
+// what pipe_poisson_solve_noalloc holds against its fixed array
+size_t mode_noalloc_bytes(const pipe_handle* h);
+// partial projections that the projection writes (groups of x rows)
 int mode_xblocks(const pipe_handle* h);
 // the FP32 mode-form arguments of a handle with its own scratch as part /
 // psi (rho, phi null): the batched call's grouped launches

@@ -65,7 +65,6 @@ namespace {
 
 template <typename T>
 cudaError_t launch_band(const ModeArgs<T>& a, cudaStream_t st) {
-  const int xblocks = a.nx / ModeShape<T>::XB;
   const size_t smem = sizeof(T) * (size_t(a.nz) + 3 * size_t(a.nb) + 1);
   void (*kern)(ModeArgs<T>, int) = mode_band_kernel<T>;
   if (smem > 48 * 1024) {
@@ -73,7 +72,7 @@ cudaError_t launch_band(const ModeArgs<T>& a, cudaStream_t st) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
   }
-  kern<<<unsigned(a.mc), kBandThreads, smem, st>>>(a, xblocks / mode_cluster(xblocks));
+  kern<<<unsigned(a.mc), kBandThreads, smem, st>>>(a, a.groups);
   return cudaGetLastError();
 }
 
@@ -122,28 +121,23 @@ cudaError_t launch_pb2(int which, bool fy, const ModeArgs<T>& a, cudaStream_t st
 
 }  // namespace
 
-#ifndef PP_M_TYPE
-#define PP_M_TYPE float
-#endif
+template <typename T>
+cudaError_t launch_mode_z_stage(const ModeArgs<T>& a, cudaStream_t st) {
+  if (a.nz < 32 || a.nz > 1024 || (a.nz & (a.nz - 1))) return cudaErrorInvalidValue;
+  return a.nb >= 0 ? launch_band<T>(a, st) : launch_mode_z<T>(a, a.groups, st);
+}
+template cudaError_t launch_mode_z_stage<float>(const ModeArgs<float>&, cudaStream_t);
+template cudaError_t launch_mode_z_stage<double>(const ModeArgs<double>&, cudaStream_t);
 
-template <>
-cudaError_t launch_mode_stage<PP_M_TYPE>(int stage, int myp, bool fy, const ModeArgs<PP_M_TYPE>& a,
-                                         cudaStream_t st) {
-  using T = PP_M_TYPE;
-  if (stage == 1) {
-    if (a.nz < 32 || a.nz > 1024 || (a.nz & (a.nz - 1))) return cudaErrorInvalidValue;
-    if (a.nb >= 0) return launch_band<T>(a, st);
-    const int xblocks = a.nx / ModeShape<T>::XB;
-    return launch_mode_z<T>(a, xblocks / mode_cluster(xblocks), st);
-  }
+cudaError_t launch_mode_sums(int stage, int myp, bool fy, const ModeArgs<float>& a, cudaStream_t st) {
   const int which = stage == 0 ? 0 : 1;
   switch (myp) {
-    case 8: return launch_pb2<T, 8>(which, fy, a, st);
-    case 12: return launch_pb2<T, 12>(which, fy, a, st);
-    case 16: return launch_pb2<T, 16>(which, fy, a, st);
-    case 20: return launch_pb2<T, 20>(which, fy, a, st);
-    case 24: return launch_pb2<T, 24>(which, fy, a, st);
-    case 32: return launch_pb2<T, 32>(which, fy, a, st);
+    case 8: return launch_pb2<float, 8>(which, fy, a, st);
+    case 12: return launch_pb2<float, 12>(which, fy, a, st);
+    case 16: return launch_pb2<float, 16>(which, fy, a, st);
+    case 20: return launch_pb2<float, 20>(which, fy, a, st);
+    case 24: return launch_pb2<float, 24>(which, fy, a, st);
+    case 32: return launch_pb2<float, 32>(which, fy, a, st);
     default: return cudaErrorInvalidValue;
   }
 }

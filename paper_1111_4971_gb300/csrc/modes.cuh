@@ -88,10 +88,12 @@ inline int mode_cluster(int xblocks) {
 constexpr int kModeZRun = 8;
 constexpr int kModeZPar = 12;
 
-// stage 0: projection rho -> part, 1: z convolution part -> psi,
-// 2: back-projection psi -> phi
+// stage 1, part -> psi: the z convolution, or the banded operator's stencil
 template <typename T>
-cudaError_t launch_mode_stage(int stage, int myp, bool fy, const ModeArgs<T>& a, cudaStream_t st);
+cudaError_t launch_mode_z_stage(const ModeArgs<T>& a, cudaStream_t st);
+// FP32 stage 0 (projection rho -> part) or 2 (back-projection psi -> phi) on
+// any mesh (FP64: modes_split.cuh)
+cudaError_t launch_mode_sums(int stage, int myp, bool fy, const ModeArgs<float>& a, cudaStream_t st);
 
 // A group of FP32 mode-form solves of one shape (nx, ny, nz, mode layout)
 // and one y-mode table, run by one launch per stage (the batched call):

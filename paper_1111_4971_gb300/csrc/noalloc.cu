@@ -69,7 +69,7 @@ extern "C" int pipe_poisson_solve_noalloc(pipe_handle* h, const void* rho, void*
   if (h->banded >= 0 || h->grid.dtype == PIPE_F32_C16) return PIPE_EUNSUPPORTED;
   if (!h->use_modes && (h->general || !h->fft_ok)) return PIPE_EUNSUPPORTED;
   const size_t cbytes = h->grid.dtype == PIPE_F64 ? 16 : 8;
-  const size_t need = h->use_modes ? pp::mode_scratch_bytes(h)
+  const size_t need = h->use_modes ? pp::mode_noalloc_bytes(h)
                                    : size_t(h->grid.nz + 1) * h->grid.nx * h->grid.ny * cbytes;
   if (need > kNoAllocScratchBytes) return PIPE_EUNSUPPORTED;     // larger than the fixed array
   int prev = -1;
