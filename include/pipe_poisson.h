@@ -178,9 +178,9 @@ int pipe_poisson_adjoint(pipe_handle* h, const void* dphi, void* drho, void* str
  * library instead of device memory owned by the handle -- for the
  * padded-transform form the z half-spectrum, (nz+1)*nx*ny complex values of
  * the dtype; for the mode-space form (plan t_kind 3) the projections and the
- * convolved mode columns, (xblocks+1)*mxp*myp*nz values (pipe_mode_layout;
- * for FP64, with xblocks taken as nx/8 over the largest divisor of nx/8 that
- * is at most 4, and never less than the scratch stated at pipe_green_setup).
+ * convolved mode columns, (xblocks+1)*mxp*myp*nz values with xblocks taken as
+ * nx/16 (FP64: nx/8) over the largest divisor of that which is at most 4, and
+ * never less than the scratch stated at pipe_green_setup.
  * The handle's current form runs, so the result is bit for bit that of
  * pipe_poisson_solve.  Meant for programs that must not let a library
  * allocate device memory while they run (a host that keeps the GPU's memory
@@ -329,14 +329,14 @@ int pipe_stage_z_inverse(pipe_handle* h, const void* spec, void* phi, int adjoin
 /* Layout of the mode-space form (Sec. 2 Eq. 7: the sine modes of the
  * truncated series).  mx = modes_m; mxp = mx rounded up to a multiple of 4;
  * myp = the y-mode slots: when the mesh is symmetric about the pipe's
- * mid-plane in y (2*y0 + (ny-1)*hy == b, e.g. cell-centred; for FP64 also
- * y0 == 0 and ny*hy == b, the first row on the wall), *fold = 1 and
+ * mid-plane in y (2*y0 + (ny-1)*hy == b, e.g. cell-centred, or y0 == 0 and
+ * ny*hy == b, the first row on the wall), *fold = 1 and
  * slot s < myp/2 holds mode n = 2s+1, slot s >= myp/2 mode n = 2(s - myp/2)+2;
  * otherwise *fold = 0 and slot s holds n = s+1 (slots beyond modes_n are
  * zero).  Mode column c = (m-1)*myp + slot.  xblocks: the groups of x rows
- * whose projections the first stage writes separately (FP32: the kernel works
- * on blocks of 16 rows and sums up to 4 neighbouring blocks in a thread-block
- * cluster; xblocks = blocks / that cluster size, 2 for nx = 128.  FP64: 1).  Errors: PIPE_EINVAL (null pointers), PIPE_EUNSUPPORTED
+ * whose projections the first stage writes separately, equal and in order
+ * (FP32: one per 8 or 16 rows on small meshes, 4 to 8 on large ones, 8 for
+ * 128^2 x 1024.  FP64: 1).  Errors: PIPE_EINVAL (null pointers), PIPE_EUNSUPPORTED
  * (the mode-space form cannot take the handle). */
 int pipe_mode_layout(pipe_handle* h, int* mx, int* mxp, int* myp, int* fold, int* xblocks);
 

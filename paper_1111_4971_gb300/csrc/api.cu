@@ -130,7 +130,6 @@ void free_handle(pipe_handle* h) {
   cudaFree(h->mwork);
   cudaFree(h->msplit);
   cudaFree(h->mkb64); cudaFree(h->mkb32);
-  std::free(h->msy_host);
   for (int k = 0; k < 2; ++k) {
     cudaFree(h->ring_rho[k]);
     cudaFree(h->ring_phi[k]);
@@ -248,8 +247,7 @@ int finish_setup(pipe_handle* h, pipe_handle** out) {
 namespace pp {
 int mode_xblocks(const pipe_handle* h) {
   if (h->grid.dtype == PIPE_F64) return 1;
-  const int xb = h->grid.nx / ModeShape<float>::XB;
-  return xb / mode_cluster(xb);
+  return mode_shape(h->grid.nx, h->grid.nz, h->mxp * h->myp).groups;
 }
 
 size_t mode_scratch_bytes(const pipe_handle* h) {
@@ -259,16 +257,14 @@ size_t mode_scratch_bytes(const pipe_handle* h) {
          (f64 ? split_half_bytes(h->grid.nx, h->myp, h->grid.nz) : 0);
 }
 
-// the scratch, but FP64 at least one partial projection per cluster of 8-row
-// blocks, the size that this entry point's documented limit stands for
+// the scratch, but at least one partial projection per up to 4 blocks of 16
+// (FP64: 8) rows, the size that this entry point's documented limit stands for
 size_t mode_noalloc_bytes(const pipe_handle* h) {
-  size_t need = mode_scratch_bytes(h);
-  if (h->grid.dtype == PIPE_F64) {
-    const int xb = h->grid.nx / 8;
-    const size_t limit = sizeof(double) * size_t(xb / mode_cluster(xb) + 1) * h->mxp * h->myp * h->grid.nz;
-    if (limit > need) need = limit;
-  }
-  return need;
+  const bool f64 = h->grid.dtype == PIPE_F64;
+  const int xb = h->grid.nx / (f64 ? 8 : 16);
+  const size_t limit = (f64 ? 8 : 4) * size_t(xb / divisor_to_4(xb) + 1) * h->mxp * h->myp * h->grid.nz;
+  const size_t need = mode_scratch_bytes(h);
+  return limit > need ? limit : need;
 }
 
 template <typename T>
@@ -287,6 +283,8 @@ ModeArgs<T> mode_args(const pipe_handle* h, const void* rho, void* phi, void* pa
   a.mxp = h->mxp;
   a.mc = h->mxp * h->myp;
   a.groups = mode_xblocks(h);
+  a.mirror = h->fy == 2 ? h->grid.ny : h->grid.ny - 1;
+  a.wall = h->fy == 2 ? h->grid.ny / 2 : 0;
   a.kb = reinterpret_cast<const T*>(D ? static_cast<const void*>(h->mkb64) : static_cast<const void*>(h->mkb32));
   a.nb = h->banded;
   return a;
@@ -299,7 +297,6 @@ int mode_stage(const pipe_handle* h, int stage, const void* rho, void* phi, void
   const ModeArgs<T> a = mode_args<T>(h, rho, phi, part, psi);
   if (stage == 1) return status_of(launch_mode_z_stage<T>(a, st));
   if constexpr (sizeof(T) == 4) {
-    if (h->mfast) return status_of(launch_mode_fast(stage, h->myp, a, h->msy_host, st));
     return status_of(launch_mode_sums(stage, h->myp, h->fy != 0, a, st));
   } else {
     SplitArgs s{};
@@ -461,9 +458,8 @@ static int setup_pipe(const pipe_geometry* geom, const pipe_grid* grid, int igf,
   s.modes_m = geom->modes_m; s.modes_n = geom->modes_n;
   s.igf = igf;
   if (modes_ok) {
-    // FP64 also folds meshes with row 0 on the wall (y_{ny-j} = b - y_j)
-    const bool wall = grid->dtype == PIPE_F64 && geom->y0 == 0.0 &&
-                      std::fabs(grid->ny * grid->hy - geom->b) <= 1e-12 * geom->b;
+    // meshes with row 0 on the wall fold too (y_{ny-j} = b - y_j)
+    const bool wall = geom->y0 == 0.0 && std::fabs(grid->ny * grid->hy - geom->b) <= 1e-12 * geom->b;
     h->fy = fold ? 1 : (wall ? 2 : 0);
     h->mxp = (geom->modes_m + 3) / 4 * 4;
     h->myp = mode_slots(geom->modes_n, h->fy != 0);
@@ -519,15 +515,6 @@ static int setup_pipe(const pipe_geometry* geom, const pipe_grid* grid, int igf,
         free_handle(h);
         return status_of(e);
       }
-    }
-    if (grid->dtype == PIPE_F32 && mode_fast_ok(grid->ny, grid->nx, h->myp, fold)) {
-      h->msy_host = static_cast<float*>(std::malloc(nsy * sizeof(float)));
-      if (!h->msy_host) { free_handle(h); return PIPE_ENOMEM; }
-      if ((e = cudaMemcpy(h->msy_host, h->msy32, nsy * sizeof(float), cudaMemcpyDeviceToHost)) != cudaSuccess) {
-        free_handle(h);
-        return status_of(e);
-      }
-      h->mfast = 1;
     }
     // the default: the mode-space form where the modes are at most half the
     // transverse mesh (or where the padded transforms cannot take the mesh)

@@ -21,7 +21,7 @@
 //
 // The solves left outside the persistent launch run as their own launches,
 // on the caller's stream or dealt to side streams.  FP32 mode-space solves of
-// one shape and one y-mode table among them can run as a group: one launch
+// one shape among them can run as a group: one launch
 // per stage (projection, z convolution, back-projection) for up to 64 solves,
 // each CTA finding its solve from its block index.  A stage of many solves is
 // a grid of many waves, so the reduction phase of some CTAs overlaps the
@@ -244,8 +244,8 @@ int z_cols(int nz) {
   return 0;
 }
 
-// FP32 mode-form solves outside the persistent launch that share a shape and
-// a y-mode table: one launch per stage for all of them (ModeGroup), the same
+// FP32 mode-form solves outside the persistent launch that share a shape: one
+// launch per stage for all of them (ModeGroup), the same
 // kernels and arithmetic per solve as their single-solve launches
 struct MGroup {
   std::vector<int> members;            // indices into the handle set
@@ -253,7 +253,7 @@ struct MGroup {
   ModeArgs<float> a0{};                // the shape (members[0]'s arguments)
   int myp = 0;
   int zgroups = 0;                     // partial projections the z stage sums
-  const float* sy = nullptr;           // the shared y-mode table (host copy)
+  bool fold = false;
 };
 
 // One way of running a handle set: the solves in the persistent launch
@@ -514,17 +514,15 @@ static double spectrum_bytes(const pipe_handle* h) {
 }
 
 // the groups of a variant's outside solves: FP32 mode-form solves with the
-// occupancy-laid-out kernels, of one shape and one y-mode table, up to
+// of one shape, up to
 // kMaxModeGroup each; only groups of two or more are kept
 static bool mode_groupable(const pipe_handle* h) {
-  return h->grid.dtype == PIPE_F32 && h->use_modes && h->mfast && h->banded < 0 && h->msy_host;
+  return h->grid.dtype == PIPE_F32 && h->use_modes && h->banded < 0;
 }
 static bool same_mode_shape(const pipe_handle* a, const pipe_handle* b) {
-  if (a->grid.nx != b->grid.nx || a->grid.ny != b->grid.ny || a->grid.nz != b->grid.nz ||
-      a->geom.modes_m != b->geom.modes_m || a->mxp != b->mxp || a->myp != b->myp || a->fy != b->fy)
-    return false;
-  const size_t nsy = size_t(a->grid.ny / 2) * a->myp;
-  return std::memcmp(a->msy_host, b->msy_host, nsy * sizeof(float)) == 0;
+  return a->grid.nx == b->grid.nx && a->grid.ny == b->grid.ny && a->grid.nz == b->grid.nz &&
+         a->geom.modes_m == b->geom.modes_m && a->geom.modes_n == b->geom.modes_n && a->mxp == b->mxp &&
+         a->myp == b->myp && a->fy == b->fy;
 }
 static int build_mode_groups(pipe_handle* const* hs, BatchVariant* v) {
   std::vector<MGroup> gs;
@@ -547,7 +545,7 @@ static int build_mode_groups(pipe_handle* const* hs, BatchVariant* v) {
     g.a0 = args[0];
     g.myp = h0->myp;
     g.zgroups = mode_xblocks(h0);
-    g.sy = h0->msy_host;
+    g.fold = h0->fy != 0;
     if (cudaMalloc(&g.dargs, sizeof(ModeArgs<float>) * args.size()) != cudaSuccess) return PIPE_ENOMEM;
     if (cudaMemcpy(g.dargs, args.data(), sizeof(ModeArgs<float>) * args.size(), cudaMemcpyHostToDevice) !=
         cudaSuccess) {
@@ -569,9 +567,9 @@ static int run_mode_group(const MGroup& g, const void* const* rho, void* const* 
     p.rho[i] = static_cast<const float*>(rho[g.members[i]]);
     p.phi[i] = static_cast<float*>(phi[g.members[i]]);
   }
-  cudaError_t e = launch_mode_fast_group(0, g.myp, g.a0, p, g.sy, st);
+  cudaError_t e = launch_mode_sums_group(0, g.myp, g.fold, g.a0, p, st);
   if (e == cudaSuccess) e = launch_mode_z_group(g.a0, g.zgroups, p, st);
-  if (e == cudaSuccess) e = launch_mode_fast_group(2, g.myp, g.a0, p, g.sy, st);
+  if (e == cudaSuccess) e = launch_mode_sums_group(2, g.myp, g.fold, g.a0, p, st);
   return e == cudaSuccess ? PIPE_OK : PIPE_ECUDA;
 }
 

@@ -71,8 +71,6 @@ struct pipe_handle {
   // part [groups][mc][nz], then psi [mc][nz], of the dtype; FP64: then the
   // half-transformed field of a slab (modes_split.cuh)
   void* mwork = nullptr;
-  float* msy_host = nullptr;   // FP32 y-mode table in host memory (the projection's kernel parameter)
-  int mfast = 0;               // FP32 projection / back-projection in their occupancy layout
   pp::Plan plan{8, 0, 1, 256};
   pp::Plan free_plan{8, 0, 1, 256};   // transverse shape of the free-space stage
   void* batch = nullptr;       // batched work list owned by this handle

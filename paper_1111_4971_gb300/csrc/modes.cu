@@ -1,23 +1,11 @@
-// Kernels and host launchers of the mode-space solve (the method and the
-// device routines are described in modes_impl.cuh).
+// z stage of the mode-space solve (the method is described in modes_impl.cuh):
+// the banded operator's stencil, or the recurrences of modes_z.cu.
 #include <type_traits>
 
 #include "modes.cuh"
 #include "modes_impl.cuh"
 
 namespace pp {
-
-template <typename T, int MYP, bool FY>
-__global__ void __launch_bounds__(128) mode_project_kernel(ModeArgs<T> a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  mode_project<T, MYP, FY>(a, smem_raw);
-}
-
-template <typename T, int MYP, bool FY>
-__global__ void __launch_bounds__(128) mode_back_kernel(ModeArgs<T> a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  mode_back<T, MYP, FY>(a, smem_raw);
-}
 
 // Banded z stage (Sec. 5, Eq. 17-18 in mode space): psi[c][k] =
 // sum_{|d| <= nb, 0 <= k-d < nz} K_c(|d|) rhot[c][k-d], rhot the groups' partial
@@ -76,49 +64,6 @@ cudaError_t launch_band(const ModeArgs<T>& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-template <typename K>
-cudaError_t set_smem(K kern, size_t smem) {
-  if (smem > kMaxSmem) return cudaErrorInvalidConfiguration;
-  if (smem <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-}
-
-template <typename T, int MYP, bool FY>
-cudaError_t launch_pb(int which, const ModeArgs<T>& a, cudaStream_t st) {
-  using S = ModeShape<T>;
-  const int xblocks = a.nx / S::XB;
-  const dim3 grid(unsigned(a.nz / S::ZC), unsigned(xblocks));
-  cudaError_t e;
-  if (which == 0) {
-    const size_t smem = mode_proj_smem<T>(a.ny, a.mxp, MYP, FY);
-    void (*kern)(ModeArgs<T>) = mode_project_kernel<T, MYP, FY>;
-    if ((e = set_smem(kern, smem)) != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(S::THREADS, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 1;
-    attr[0].val.clusterDim.y = unsigned(mode_cluster(xblocks));
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, a);
-  }
-  const size_t smem = mode_back_smem<T>(a.ny, a.mx, a.mxp, MYP, FY);
-  void (*kern)(ModeArgs<T>) = mode_back_kernel<T, MYP, FY>;
-  if ((e = set_smem(kern, smem)) != cudaSuccess) return e;
-  kern<<<grid, S::THREADS, smem, st>>>(a);
-  return cudaGetLastError();
-}
-
-template <typename T, int MYP>
-cudaError_t launch_pb2(int which, bool fy, const ModeArgs<T>& a, cudaStream_t st) {
-  return fy ? launch_pb<T, MYP, true>(which, a, st) : launch_pb<T, MYP, false>(which, a, st);
-}
-
 }  // namespace
 
 template <typename T>
@@ -128,18 +73,5 @@ cudaError_t launch_mode_z_stage(const ModeArgs<T>& a, cudaStream_t st) {
 }
 template cudaError_t launch_mode_z_stage<float>(const ModeArgs<float>&, cudaStream_t);
 template cudaError_t launch_mode_z_stage<double>(const ModeArgs<double>&, cudaStream_t);
-
-cudaError_t launch_mode_sums(int stage, int myp, bool fy, const ModeArgs<float>& a, cudaStream_t st) {
-  const int which = stage == 0 ? 0 : 1;
-  switch (myp) {
-    case 8: return launch_pb2<float, 8>(which, fy, a, st);
-    case 12: return launch_pb2<float, 12>(which, fy, a, st);
-    case 16: return launch_pb2<float, 16>(which, fy, a, st);
-    case 20: return launch_pb2<float, 20>(which, fy, a, st);
-    case 24: return launch_pb2<float, 24>(which, fy, a, st);
-    case 32: return launch_pb2<float, 32>(which, fy, a, st);
-    default: return cudaErrorInvalidValue;
-  }
-}
 
 }  // namespace pp

@@ -8,52 +8,20 @@ namespace pp {
 template <typename T>
 struct ModeArgs;
 
-// tile shape of the projection and back-projection kernels
+// The mode form takes a mesh where these two are within a CTA's shared memory:
+// the sizes of a projection and a back-projection kernel that stage a ring of
+// field rows, the y-mode table and 32 z values of the mode columns.
 template <typename T>
-struct ModeShape {
-  static constexpr int WARPS = 4;
-  static constexpr int THREADS = 32 * WARPS;
-  static constexpr int ZC = 32;                              // z values per CTA, one per lane
-  static constexpr int XPW = sizeof(T) == 4 ? 4 : 2;         // x rows per warp
-  static constexpr int XB = WARPS * XPW;                     // x rows per CTA
-  static constexpr int YK = 4;                               // y rows per stage (and their mirrors)
-  static constexpr int STAGES = 3;
-  static constexpr int MQ = sizeof(T) == 4 ? 4 : 2;          // x modes per pass of the projection
-  // the projection's x modes in this many rounds, each summed over the
-  // cluster before the next: the block's projection buffer holds one round
-  // (FP64: half the modes, so that two CTAs fit in an SM's shared memory)
-  static constexpr int RED_PASSES = sizeof(T) == 4 ? 1 : 2;
-};
-
-// x modes of one round of the projection (a multiple of MQ)
-template <typename T>
-__host__ __device__ inline int mode_round_modes(int mxp) {
-  using S = ModeShape<T>;
-  return (mxp + S::RED_PASSES * S::MQ - 1) / (S::RED_PASSES * S::MQ) * S::MQ;
-}
-
-// shared memory of the projection (elements): the ring of row stages, which
-// after the y loop holds the y-mode sums [XB][myp][ZC] and one round of the
-// block's projection [mode_round_modes * myp][ZC]; then the y-mode table and
-// the block's x rows
-template <typename T>
-__host__ __device__ inline size_t mode_proj_union(int mxp, int myp, bool fy) {
-  using S = ModeShape<T>;
-  const size_t slab = size_t(S::STAGES) * S::XB * (fy ? 2 * S::YK : S::YK) * S::ZC;
-  const size_t after = size_t(S::XB) * myp * S::ZC + size_t(mode_round_modes<T>(mxp)) * myp * S::ZC;
-  return slab > after ? slab : after;
+inline size_t mode_proj_smem(int ny, int mxp, int myp, bool fold) {
+  constexpr int XB = sizeof(T) == 4 ? 16 : 8, ZC = 32;
+  const int mpass = sizeof(T) == 4 ? mxp : (mxp + 3) / 4 * 2;          // FP64: the x modes in two rounds
+  const size_t ring = size_t(3) * XB * (fold ? 8 : 4) * ZC, sums = size_t(XB + mpass) * myp * ZC;
+  return sizeof(T) * ((ring > sums ? ring : sums) + size_t(fold ? ny / 2 : ny) * myp + size_t(XB) * mxp);
 }
 template <typename T>
-__host__ __device__ inline size_t mode_proj_smem(int ny, int mxp, int myp, bool fy) {
-  return sizeof(T) * (mode_proj_union<T>(mxp, myp, fy) + size_t(fy ? ny / 2 : ny) * myp +
-                      size_t(ModeShape<T>::XB) * mxp);
-}
-// shared memory of the back-projection: the psi chunk [mx * myp][ZC], the
-// y-mode table, the block's x rows
-template <typename T>
-__host__ __device__ inline size_t mode_back_smem(int ny, int mx, int mxp, int myp, bool fy) {
-  return sizeof(T) * (size_t(mx) * myp * ModeShape<T>::ZC + size_t(fy ? ny / 2 : ny) * myp +
-                      size_t(ModeShape<T>::XB) * mxp);
+inline size_t mode_back_smem(int ny, int mx, int mxp, int myp, bool fold) {
+  constexpr int XB = sizeof(T) == 4 ? 16 : 8, ZC = 32;
+  return sizeof(T) * (size_t(mx) * myp * ZC + size_t(fold ? ny / 2 : ny) * myp + size_t(XB) * mxp);
 }
 
 // y-mode slots of the tables (MYP, a multiple of 4 in {8, 12, 16, 20, 24, 32}):
@@ -72,15 +40,45 @@ inline int mode_of_slot(int s, int myp, bool fold) {
   return s < myp / 2 ? 2 * s + 1 : 2 * (s - myp / 2) + 2;
 }
 
-// CTAs per cluster of the projection: the largest divisor of its x blocks
-// that is at most 4; the projection writes xblocks / mode_cluster(xblocks)
-// partial sums, which the z convolution adds on load.  (Clusters of 8, one
-// partial at 128 x rows, kept every CTA in the distributed-shared-memory
-// reduction longer than the second partial costs the z kernel.)
-inline int mode_cluster(int xblocks) {
+// the largest divisor of n that is at most 4
+inline int divisor_to_4(int n) {
   for (int d = 4; d > 1; --d)
-    if (xblocks % d == 0) return d;
+    if (n % d == 0) return d;
   return 1;
+}
+
+// Shape of the FP32 projection and back-projection (modes_sums.cu): warps per
+// CTA (of kModeRowsPerWarp x rows each), and of the projection the x blocks that
+// a CTA takes one after the other (reps) and the groups of them, each writing
+// one partial.
+//   Warps: 8, or 4 where 8 leave fewer than 128 CTAs (64^2 x 256, 8 / 4 warps:
+//   projection 7.2 / 7.3, back-projection 6.5 / 5.9 us; 128^2 x 1024, 8 / 4 / 16:
+//   20.3 / 21.9 / 31.6 and 17.5 / 18.1 / 17.1).  One x row a warp: 25.8 and 23.7.
+//   Groups: every x block its own while there are at most 16 (128^2 x 1024, 8 / 4
+//   groups: 20.3 / 23.5 us), else a divisor of 4 to 8: the partials (1.6 MB each
+//   at 400 columns of 1024) would come near the field's own bytes.  Their memory
+//   is at most 48 MiB, or what one partial per up to 4 blocks of 16 rows takes.
+constexpr int kModeRowsPerWarp = 2;
+struct ModeShape {
+  int warps, reps, groups;
+};
+inline ModeShape mode_shape(int nx, int nz, int columns) {
+  ModeShape s{};
+  s.warps = nz / 32 * nx / (8 * kModeRowsPerWarp) < 128 ? 4 : 8;
+  const int xblocks = nx / (s.warps * kModeRowsPerWarp), xb16 = nx / 16;
+  const size_t partial = sizeof(float) * size_t(columns) * nz, most = size_t(48) << 20;
+  const size_t old = size_t(xb16 / divisor_to_4(xb16) + 1) * partial, cap = old > most ? old : most;
+  s.groups = xblocks;
+  if (xblocks > 16) {
+    int g = 8;
+    while (g >= 4 && xblocks % g) --g;
+    for (int k = 9; g < 4 && k <= xblocks; ++k)
+      if (xblocks % k == 0) { g = k; break; }
+    s.groups = g;
+  }
+  while (s.groups > 1 && (xblocks % s.groups || size_t(s.groups + 1) * partial > cap)) --s.groups;
+  s.reps = xblocks / s.groups;
+  return s;
 }
 
 // z recurrences (modes_z.cu): z values per thread, and the parameters of a
@@ -92,11 +90,11 @@ constexpr int kModeZPar = 12;
 template <typename T>
 cudaError_t launch_mode_z_stage(const ModeArgs<T>& a, cudaStream_t st);
 // FP32 stage 0 (projection rho -> part) or 2 (back-projection psi -> phi) on
-// any mesh (FP64: modes_split.cuh)
-cudaError_t launch_mode_sums(int stage, int myp, bool fy, const ModeArgs<float>& a, cudaStream_t st);
+// any mesh (modes_sums.cu; FP64: modes_split.cuh)
+cudaError_t launch_mode_sums(int stage, int myp, bool fold, const ModeArgs<float>& a, cudaStream_t st);
 
-// A group of FP32 mode-form solves of one shape (nx, ny, nz, mode layout)
-// and one y-mode table, run by one launch per stage (the batched call):
+// A group of FP32 mode-form solves of one shape (nx, ny, nz, mode layout),
+// run by one launch per stage (the batched call):
 // args[s] (device memory) holds solve s's tables and scratch, rho / phi its
 // field arrays (kernel parameters, so that a captured launch keeps them).
 constexpr int kMaxModeGroup = 64;
@@ -115,12 +113,8 @@ cudaError_t launch_mode_z(const ModeArgs<T>& a, int groups, cudaStream_t st);
 // the same for a group (columns of solve s in the CTAs s * cps ..)
 cudaError_t launch_mode_z_group(const ModeArgs<float>& a, int groups, const ModeGroup& g, cudaStream_t st);
 
-// the FP32 projection and back-projection laid out for occupancy
-// (modes_fast.cu): meshes symmetric in y with ny/2 in {16, 32, 64, 128}
-bool mode_fast_ok(int ny, int nx, int myp, bool fy);
-// sy_host: the FP32 y-mode table [ny/2][myp] in host memory (the projection's parameter)
-cudaError_t launch_mode_fast(int stage, int myp, const ModeArgs<float>& a, const float* sy_host, cudaStream_t st);
-cudaError_t launch_mode_fast_group(int stage, int myp, const ModeArgs<float>& a, const ModeGroup& g,
-                                   const float* sy_host, cudaStream_t st);
+// launch_mode_sums for a group (g->args[s] shaped like a)
+cudaError_t launch_mode_sums_group(int stage, int myp, bool fold, const ModeArgs<float>& a, const ModeGroup& g,
+                                   cudaStream_t st);
 
 }  // namespace pp

@@ -61,10 +61,13 @@ __device__ __forceinline__ void z_scan(const ModeArgs<T>& a, int groups, int blk
   const T beta = par[0], gamma = par[1], p = sizeof(T) == 4 ? par[2] : par[3];
   const T* w = par + 4;                           // w[i] = q^{kV 2^i}
 
-  // the column's values, summed over the groups of partial projections
-  T x[kV];
+  wait_stage();
+  // the column's values, the groups of partial projections summed with the
+  // rounding errors of the additions carried along (Knuth's TwoSum): the partial
+  // sums of a density that changes sign can cancel
+  T x[kV], c[kV];
 #pragma unroll
-  for (int j = 0; j < kV; ++j) x[j] = T(0);
+  for (int j = 0; j < kV; ++j) x[j] = c[j] = T(0);
   if (valid) {
 #pragma unroll 8
     for (int s = 0; s < groups; ++s) {
@@ -73,9 +76,15 @@ __device__ __forceinline__ void z_scan(const ModeArgs<T>& a, int groups, int blk
 #pragma unroll
       for (int i = 0; i < kV / EV; ++i) *reinterpret_cast<V*>(g + EV * i) = __ldg(src + i);
 #pragma unroll
-      for (int j = 0; j < kV; ++j) x[j] += g[j];
+      for (int j = 0; j < kV; ++j) {
+        const T sum = x[j] + g[j], d = sum - x[j];
+        if (sizeof(T) == 4) c[j] += (x[j] - (sum - d)) + (g[j] - d);      // FP64 writes one partial
+        x[j] = sum;
+      }
     }
   }
+#pragma unroll
+  for (int j = 0; j < kV; ++j) x[j] += c[j];
   // totals of the thread's values, then of all threads up to this one
   T sf = x[0], sb = x[kV - 1];
 #pragma unroll
@@ -150,12 +159,10 @@ cudaError_t launch_z_nz(const ModeArgs<T>& a, int groups, const ModeGroup* g, cu
   const int cps = (a.mc + per - 1) / per;         // CTAs per solve
   if constexpr (sizeof(T) == 4) {
     if (g) {
-      mode_z_group_kernel<NZ><<<g->n * cps, kZThreads, 0, st>>>(*g, groups, cps);
-      return cudaGetLastError();
+      return launch_stage(mode_z_group_kernel<NZ>, dim3(unsigned(g->n * cps)), kZThreads, 0, st, *g, groups, cps);
     }
   }
-  mode_z_kernel<T, NZ><<<cps, kZThreads, 0, st>>>(a, groups);
-  return cudaGetLastError();
+  return launch_stage(mode_z_kernel<T, NZ>, dim3(unsigned(cps)), kZThreads, 0, st, a, groups);
 }
 
 template <typename T>
