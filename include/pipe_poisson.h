@@ -116,9 +116,10 @@ typedef struct pipe_handle pipe_handle;
  *    (FP64 about 10 times that, as fragments for the tensor cores) and its
  *    scratch (xblocks + 1)*mxp*myp*nz values of the dtype (the sizes of
  *    pipe_mode_layout); FP64 in addition nx*myp*nz values, at most 32 MiB.
- *    The default where the modes are at most half the transverse mesh
- *    (2*max(ceil4(modes_m), slots) <= min(nx, ny)) or the padded transforms
- *    cannot take the mesh.
+ *    The default in FP64, where the padded transforms cannot take the mesh,
+ *    where the modes are at most half the transverse mesh
+ *    (2*max(ceil4(modes_m), slots) <= min(nx, ny)), and up to 24 modes on
+ *    meshes of at least 512 nodes per mode pair.
  * A mesh that neither form takes gives PIPE_EUNSUPPORTED.
  * Errors: PIPE_EINVAL (non-positive sizes or spacings, mesh not inside the
  * pipe, bad dtype / igf, out == NULL), PIPE_EUNSUPPORTED (other sizes or

@@ -516,10 +516,17 @@ static int setup_pipe(const pipe_geometry* geom, const pipe_grid* grid, int igf,
         return status_of(e);
       }
     }
-    // the default: the mode-space form where the modes are at most half the
-    // transverse mesh (or where the padded transforms cannot take the mesh)
-    const int nmin = grid->nx < grid->ny ? grid->nx : grid->ny;
-    h->use_modes = (!fft_ok || 2 * (h->mxp > h->myp ? h->mxp : h->myp) <= nmin) ? 1 : 0;
+    // the default: the mode-space form in FP64 (exact products on the tensor
+    // cores against transforms on the FP64 pipe: 16^2 x 32 30 against 49 us,
+    // 32^2 x 1024 54 / 545) and where the padded transforms cannot take the
+    // mesh; in FP32 where the modes are at most half the transverse mesh, and
+    // up to 24 modes on meshes of at least 512 nodes a mode pair (20 modes, form
+    // against form in a captured graph: 16^2 x 256 11.7 / 10.0, 16^2 x 1024
+    // 13.1 / 17.2, 32^2 x 64 14.0 / 11.3, 32^2 x 256 14.0 / 15.2, 32^2 x 1024
+    // 14.7 / 35.6 us; 32 modes: 32^2 x 256 22.1 / 15.1)
+    const int nmin = grid->nx < grid->ny ? grid->nx : grid->ny, mmax = h->mxp > h->myp ? h->mxp : h->myp;
+    const bool long_enough = mmax <= 24 && size_t(grid->nx) * grid->ny * grid->nz >= size_t(512) * h->mxp * h->myp;
+    h->use_modes = (!fft_ok || grid->dtype == PIPE_F64 || 2 * mmax <= nmin || long_enough) ? 1 : 0;
   }
   if (!fft_ok) return finish_setup(h, out);
   // FP64 planes too large for shared memory: the n-point routine's plane

@@ -492,4 +492,28 @@ __device__ __forceinline__ void mirror_fetch(const V (&v)[GroupShape<L>::E], V (
   }
 }
 
+// Programmatic dependent launch of a stage after the one before it: it is set up
+// while that one's last CTAs run, reads tables, and calls wait_stage() before it
+// touches anything a kernel writes (the call returns when every kernel before
+// has completed and its writes are visible).  128^2 x 1024 launched one solve
+// after the other: 49.6 -> 45.5 us, 64^2 x 256 20.8 -> 17.0 us.  No stage lets
+// the next in before its CTAs end (griddepcontrol.launch_dependents): the next
+// one's CTAs then take the place of its own, 51.6 us.
+__device__ __forceinline__ void wait_stage() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename K, typename... A>
+cudaError_t launch_stage(K kern, dim3 grid, int threads, size_t smem, cudaStream_t st, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(unsigned(threads), 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 }  // namespace pp

@@ -19,6 +19,7 @@ __global__ void __launch_bounds__(kBandThreads) mode_band_kernel(ModeArgs<T> a, 
   T* win = reinterpret_cast<T*>(smem_raw);           // [nz + 2 nb]: win[nb + k] = rhot[k]
   T* taps = win + a.nz + 2 * a.nb;                   // [nb + 1]
   const int c = int(blockIdx.x);
+  wait_stage();
   for (int i = int(threadIdx.x); i < a.nb; i += kBandThreads) win[i] = win[a.nb + a.nz + i] = T(0);
   // the column summed over the groups (in group order, from zero), 16 bytes a
   // load, every group's load of a piece in flight together (nz is a power of
@@ -60,8 +61,7 @@ cudaError_t launch_band(const ModeArgs<T>& a, cudaStream_t st) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
   }
-  kern<<<unsigned(a.mc), kBandThreads, smem, st>>>(a, a.groups);
-  return cudaGetLastError();
+  return launch_stage(kern, dim3(unsigned(a.mc)), kBandThreads, smem, st, a, a.groups);
 }
 
 }  // namespace

@@ -45,8 +45,8 @@
 #include <cmath>
 #include <utility>
 
+#include "modes_impl.cuh"
 #include "modes_split.cuh"
-#include "zfft_impl.cuh"
 
 namespace pp {
 
@@ -290,6 +290,7 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 3) split_contract_kernel(con
     return 16 * ks + 8 * (i >> 1) < a.K ? *slot(ks, half, i) : make_double2(0.0, 0.0);
   };
   int unit = int(blockIdx.x) * kSplitWarps + warp, s0 = 0;
+  wait_stage();
   if (unit < units)
     for (int ks = 0; ks < min(kSeg / 16, steps); ++ks) copy(unit, ks);
 #pragma unroll 1
@@ -469,6 +470,7 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 3) split_expand_kernel(const
   double* out = a.out + size_t(o) * a.out_o + z;
   constexpr int KH = FOLD ? KS / 2 : KS;             // k steps of an accumulator
   const int kmax = FOLD ? a.K / 2 : a.K;
+  wait_stage();
   double2 x[KS][4];
   auto largest = [&]() {
     unsigned m = 0;
@@ -638,8 +640,8 @@ cudaError_t go_contract(const ContractArgs& a, cudaStream_t st) {
   const cudaError_t e = cudaFuncSetAttribute(split_contract_kernel<NT, FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   const unsigned need = units_grid(a.outer * a.ztiles), most = unsigned(3 * sm_count());   // 3 CTAs per SM
-  split_contract_kernel<NT, FOLD><<<need < most ? need : most, 32 * kSplitWarps, smem, st>>>(a);
-  return cudaGetLastError();
+  // (the first kernel of a solve, whose input others write, waits for it at once)
+  return launch_stage(split_contract_kernel<NT, FOLD>, dim3(need < most ? need : most), 32 * kSplitWarps, smem, st, a);
 }
 
 cudaError_t contract(const ContractArgs& a, bool fold, cudaStream_t st) {
@@ -655,8 +657,7 @@ cudaError_t contract(const ContractArgs& a, bool fold, cudaStream_t st) {
 
 template <typename K>
 cudaError_t go(K kern, const ExpandArgs& a, cudaStream_t st) {
-  kern<<<units_grid(a.outer * a.ztiles), 32 * kSplitWarps, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_stage(kern, dim3(units_grid(a.outer * a.ztiles)), 32 * kSplitWarps, 0, st, a);
 }
 
 cudaError_t expand(const ExpandArgs& a, bool fold, bool small, cudaStream_t st) {

@@ -124,6 +124,7 @@ __device__ __forceinline__ void project(const ModeArgs<float>& a, int zc, int gr
   const int ns = a.ny / kRows;                                 // ring stages of a row
   float* ring = abuf + warp * SL;
   const size_t nz = size_t(a.nz), xs = size_t(a.ny) * nz;
+  wait_stage();
   const int r4 = lane >> 3, piece = lane & 7;                  // this lane's row of a run of 4, 16-byte piece
 #pragma unroll 1
   for (int rep = 0; rep < reps; ++rep) {
@@ -381,8 +382,7 @@ cudaError_t launch_sums(int stage, const ModeArgs<float>& a, const ModeGroup& g,
   if (stage == 0) {
     const size_t smem = project_smem<MYP>(sh.warps, a.mxp, table);
     if ((e = big_smem(mode_project_kernel<MYP, FOLD, TS>, smem)) != cudaSuccess) return e;
-    mode_project_kernel<MYP, FOLD, TS><<<dim3(gx, unsigned(sh.groups)), 32 * sh.warps, smem, st>>>(a, g, sh.reps);
-    return cudaGetLastError();
+    return launch_stage(mode_project_kernel<MYP, FOLD, TS>, dim3(gx, unsigned(sh.groups)), 32 * sh.warps, smem, st, a, g, sh.reps);
   }
   const size_t smem = back_smem<MYP>(sh.warps, a.mx, a.mxp, table);
   if ((e = big_smem(mode_back_kernel<MYP, FOLD, TS>, smem)) != cudaSuccess) return e;

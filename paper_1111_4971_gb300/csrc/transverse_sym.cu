@@ -69,6 +69,7 @@ static cudaError_t tclaunch(const SolveArgs<T>& a, cudaStream_t st) {
 template <typename T, int N, int THREADS, bool ADJ, bool H16 = false, bool GB = false>
 __global__ void __launch_bounds__(THREADS, 1) transverse_dst_kernel(SolveArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  wait_stage();
   tdst_plane<T, N, THREADS, ADJ, H16, GB>(a, blockIdx.x, smem_raw);
 }
 
@@ -87,8 +88,7 @@ static cudaError_t tdlaunch(const SolveArgs<T>& a, cudaStream_t st) {
       cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
       if (e != cudaSuccess) return e;
     }
-    kern<<<a.nz + 1, THREADS, smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_stage(kern, dim3(unsigned(a.nz + 1)), THREADS, smem, st, a);
   }
 }
 

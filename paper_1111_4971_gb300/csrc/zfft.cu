@@ -21,6 +21,7 @@ __device__ __forceinline__ int next_wave_tile() {
 template <typename T, int NZ, int WARPS, bool CONJ, bool H16>
 __global__ void __launch_bounds__(32 * WARPS, z_ctas_per_sm<WARPS>()) zfwd_kernel(SolveArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  wait_stage();
   if (threadIdx.x == 0) {
     // its input columns (contiguous, whole 16-byte units) into L2
     using Cfg = ZCfg<T, NZ, WARPS>;
@@ -38,6 +39,7 @@ __global__ void __launch_bounds__(32 * WARPS, z_ctas_per_sm<WARPS>()) zfwd_kerne
 template <typename T, int NZ, int WARPS, bool CONJ, bool H16>
 __global__ void __launch_bounds__(32 * WARPS, z_ctas_per_sm<WARPS>()) zinv_kernel(SolveArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  wait_stage();
   zinv_tile<T, NZ, WARPS, CONJ, H16>(a, blockIdx.x, smem_raw);
 }
 
@@ -91,8 +93,7 @@ static cudaError_t zlaunch(bool forward, const SolveArgs<T>& a, cudaStream_t st)
     if (e != cudaSuccess) return e;
   }
   const int ncols = a.nx * a.ny;
-  kern<<<(ncols + Cfg::COLS - 1) / Cfg::COLS, Cfg::THREADS, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_stage(kern, dim3(unsigned((ncols + Cfg::COLS - 1) / Cfg::COLS)), Cfg::THREADS, smem, st, a);
 }
 
 template <typename T, int NZ, int W>
