@@ -440,6 +440,10 @@ int pipe_electric_field(pipe_handle* h, const void* phi, void* E, void* stream);
 int pipe_cic_deposit(pipe_handle* h, const void* xyz, int64_t n, double q, void* rho,
                      void* stream);
 
+/* pipe_cic_deposit into a field that the call clears first (on the stream):
+ * rho = the deposit.  Same arguments and errors; xyz may be null for n = 0. */
+int pipe_cic_deposit_new(pipe_handle* h, const void* xyz, int64_t n, double q, void* rho, void* stream);
+
 /* Adjoint of the deposit with respect to the positions: for a cotangent
  * grad_rho on the mesh, grad_xyz[p][d] = q/(hx*hy*hz) * sum_nodes grad_rho *
  * d w / d x_d  (derivative of the trilinear weights).  Device arrays. */

@@ -23,14 +23,21 @@ __all__ = ["PipeSolver", "PipePoissonFunction", "CICDeposit", "solve_batched", "
            "batch_select_streams", "batch_grouped", "batch_select_groups", "PipeError", "field_energy"]
 
 
+# The raw handle of a device's current stream, without building a Stream object
+# (3.0 us of a 13 us call on a Grace core).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream_ptr(stream):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _ptr(t: torch.Tensor):
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _spans(geometry, grid) -> bool:
@@ -250,8 +257,12 @@ class PipeSolver:
 
     def cic_deposit(self, xyz: torch.Tensor, charge: float, out: torch.Tensor | None = None,
                     stream=None):
-        out = torch.zeros(self.shape, dtype=self.dtype, device=self.device) if out is None else out
         xyz = xyz.contiguous()
+        if out is None:                          # cleared by the call, on its stream
+            out = self.empty()
+            check(self.lib.pipe_cic_deposit_new(self.handle, _ptr(xyz), xyz.shape[0], float(charge), _ptr(out),
+                                                _stream_ptr(stream)), "pipe_cic_deposit_new")
+            return out
         check(self.lib.pipe_cic_deposit(self.handle, _ptr(xyz), xyz.shape[0], float(charge), _ptr(out),
                                         _stream_ptr(stream)), "pipe_cic_deposit")
         return out

@@ -72,6 +72,7 @@ SIGNATURES = {
     "pipe_status": (c_int, [H]),
     "pipe_inject_stage_fault": (c_int, [H, c_int, ctypes.c_longlong]),
     "pipe_cic_deposit": (c_int, [H, c_void_p, c_int64, c_double, c_void_p, c_void_p]),
+    "pipe_cic_deposit_new": (c_int, [H, c_void_p, c_int64, c_double, c_void_p, c_void_p]),
     "pipe_cic_gather_grad": (c_int, [H, c_void_p, c_int64, c_double, c_void_p, c_void_p, c_void_p]),
     "pipe_green_destroy": (None, [H]),
     "pipe_strerror": (c_char_p, [c_int]),

@@ -143,6 +143,14 @@ extern "C" int pipe_cic_deposit(pipe_handle* h, const void* xyz, int64_t n, doub
   return cudaGetLastError() == cudaSuccess ? PIPE_OK : PIPE_ECUDA;
 }
 
+extern "C" int pipe_cic_deposit_new(pipe_handle* h, const void* xyz, int64_t n, double q, void* rho,
+                                    void* stream) {
+  if (!h || !rho || n < 0 || (n > 0 && !xyz)) return PIPE_EINVAL;
+  const size_t bytes = size_t(h->grid.nx) * h->grid.ny * h->grid.nz * (h->grid.dtype == PIPE_F64 ? 8 : 4);
+  if (cudaMemsetAsync(rho, 0, bytes, static_cast<cudaStream_t>(stream)) != cudaSuccess) return PIPE_ECUDA;
+  return n == 0 ? PIPE_OK : pipe_cic_deposit(h, xyz, n, q, rho, stream);
+}
+
 extern "C" int pipe_cic_gather_grad(pipe_handle* h, const void* xyz, int64_t n, double q,
                                     const void* grad_rho, void* grad_xyz, void* stream) {
   if (!h || !xyz || !grad_rho || !grad_xyz || n < 0) return PIPE_EINVAL;
