@@ -31,12 +31,12 @@
 //
 // Bounds, 20 x 20 modes, us per launch back to back (before: the cluster kernels
 // on ny = 32 .. 256 folded, generic 4-warp kernels elsewhere):
-//   128^2 x 1024   project 25.2 -> 19.8, back 17.8 -> 16.2  (67 MB each: 10 us);
-//                  of the projection 5 are the x-mode sums and their partials,
-//                  when every CTA of the one wave leaves the stream
-//   512^2 x 1024   project 303 -> 207, back 206 -> 162      (1.07 GB: 158 us)
-//   48 x 80 x 512  project 29.0 -> 8.6, back 12.8 -> 7.8    (window: latency)
-//   64^2 x 256     project 10.1 -> 7.3, back 8.4 -> 5.8     (latency)
+//   128^2 x 1024   project 25.2 -> 17.9, back 17.8 -> 16.3  (67 MB each: 10 us);
+//                  of the projection 3 to 4 are the x-mode sums and their
+//                  partials, when every CTA of the one wave leaves the stream
+//   512^2 x 1024   project 303 -> 201, back 206 -> 172      (1.07 GB: 158 us)
+//   48 x 80 x 512  project 29.0 -> 7.1, back 12.8 -> 7.4    (window: latency)
+//   64^2 x 256     project 10.1 -> 5.8, back 8.4 -> 5.4     (latency)
 // Ring depths of 3 to 6 stages differ by under 2 %.
 #include "modes.cuh"
 #include "modes_impl.cuh"
@@ -106,6 +106,65 @@ constexpr size_t project_smem(int warps, int mxp, int table) {
 template <int MYP>
 constexpr size_t back_smem(int warps, int mx, int mxp, int table) {
   return sizeof(float) * (size_t(mx) * MYP * kZC + warps * XR * mxp + table);
+}
+
+// P[m][n][z] = sum_x Sx[x][m] A[x][n][z] of the CTA's x rows for the slots n =
+// warp, warp + warps, .., NB at a time (the last one again where a slot is
+// missing, not stored), at most MQ quads of x modes.  Bound by the issue of the
+// broadcast loads of Sx, one per two packed FMAs of a slot: two slots at a time
+// halve them.
+template <int MYP, int MQ, int NB>
+__device__ __forceinline__ void x_modes(const float* abuf, const float* sxs, float* out, int mxp, int mq, int warps,
+                                        int rows, size_t nz, bool add) {
+  constexpr int RA = row_a<MYP>(), SL = slot_a<MYP>();
+  const int lane = threadIdx.x & 31;
+#pragma unroll 1
+  for (int n0 = int(threadIdx.x) >> 5; n0 < MYP; n0 += NB * warps) {
+    float2 p[NB][MQ][2];
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+      for (int q = 0; q < MQ; ++q) p[b][q][0] = p[b][q][1] = make_float2(0.f, 0.f);
+    const float* av = abuf + n0 * kZC + lane;
+    int step[NB];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) step[b] = n0 + b * warps < MYP ? b * warps * kZC : 0;
+#pragma unroll 2
+    for (int x = 0; x < rows; ++x) {
+      float2 v[NB];
+#pragma unroll
+      for (int b = 0; b < NB; ++b) {
+        const float f = av[(x / XR) * SL + (x % XR) * RA + step[b]];
+        v[b] = make_float2(f, f);
+      }
+      const float4* sx = reinterpret_cast<const float4*>(sxs + x * mxp);
+#pragma unroll
+      for (int q = 0; q < MQ; ++q)
+        if (q < mq) {
+          const float4 w = sx[q];
+#pragma unroll
+          for (int b = 0; b < NB; ++b) {
+            p[b][q][0] = ffma2(make_float2(w.x, w.y), v[b], p[b][q][0]);
+            p[b][q][1] = ffma2(make_float2(w.z, w.w), v[b], p[b][q][1]);
+          }
+        }
+    }
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      if (n0 + b * warps >= MYP) continue;
+#pragma unroll
+      for (int q = 0; q < MQ; ++q)
+        if (q < mq) {
+          float* d = out + size_t(4 * q * MYP + n0 + b * warps) * nz;
+          const size_t ms = MYP * nz;
+          float4 f = make_float4(p[b][q][0].x, p[b][q][0].y, p[b][q][1].x, p[b][q][1].y);
+          if (add) {                                   // the same thread's sums of the blocks before
+            f.x += d[0]; f.y += d[ms]; f.z += d[2 * ms]; f.w += d[3 * ms];
+          }
+          d[0] = f.x; d[ms] = f.y; d[2 * ms] = f.z; d[3 * ms] = f.w;
+        }
+    }
+  }
 }
 
 // z chunk zc, x blocks grp * reps ..
@@ -210,40 +269,15 @@ __device__ __forceinline__ void project(const ModeArgs<float>& a, int zc, int gr
       }
     __syncthreads();
 
-    // P[m][n][z] = sum_x Sx[x][m] A[x][n][z], the slots n warp-strided
+    // P[m][n][z]: up to 20 x modes the slots two at a time, beyond, where the sums
+    // of two take 64 registers, one by one.  Projection at 128^2 x 1024, 64^2 x
+    // 256 and 48 x 80 x 512 with 20 x modes: two at a time 17.9 / 5.8 / 7.1 us,
+    // one 18.6 / 6.1 / 7.8, three 18.6 / 7.0 / 8.4, the form of 32 x modes for
+    // all 19.6 / 6.7 / 8.1
     float* out = a.part + size_t(grp) * a.mc * nz + z0 + lane;
     const int mq = a.mxp / 4;
-#pragma unroll 1
-    for (int n = warp; n < MYP; n += kW) {
-      float2 p[8][2];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) p[q][0] = p[q][1] = make_float2(0.f, 0.f);
-      const float* av = abuf + n * kZC + lane;
-#pragma unroll 2
-      for (int x = 0; x < kX; ++x) {
-        const float f = av[(x / XR) * SL + (x % XR) * RA];
-        const float2 v = make_float2(f, f);
-        const float4* sx = reinterpret_cast<const float4*>(sxs + x * a.mxp);
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-          if (q < mq) {
-            const float4 w = sx[q];
-            p[q][0] = ffma2(make_float2(w.x, w.y), v, p[q][0]);
-            p[q][1] = ffma2(make_float2(w.z, w.w), v, p[q][1]);
-          }
-      }
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        if (q < mq) {
-          float* d = out + size_t(4 * q * MYP + n) * nz;
-          const size_t ms = MYP * nz;
-          float4 f = make_float4(p[q][0].x, p[q][0].y, p[q][1].x, p[q][1].y);
-          if (rep > 0) {                               // the same thread's sums of the blocks before
-            f.x += d[0]; f.y += d[ms]; f.z += d[2 * ms]; f.w += d[3 * ms];
-          }
-          d[0] = f.x; d[ms] = f.y; d[2 * ms] = f.z; d[3 * ms] = f.w;
-        }
-    }
+    if (mq <= 5) x_modes<MYP, 5, 2>(abuf, sxs, out, a.mxp, mq, kW, kX, nz, rep > 0);
+    else x_modes<MYP, 8, 1>(abuf, sxs, out, a.mxp, mq, kW, kX, nz, rep > 0);
     if (rep + 1 < reps) __syncthreads();               // A and the x rows read before they are refilled
   }
 }
