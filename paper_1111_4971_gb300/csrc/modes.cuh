@@ -55,7 +55,7 @@ inline int divisor_to_4(int n) {
 //   projection 7.2 / 7.3, back-projection 6.5 / 5.9 us; 128^2 x 1024, 8 / 4 / 16:
 //   20.3 / 21.9 / 31.6 and 17.5 / 18.1 / 17.1).  One x row a warp: 25.8 and 23.7.
 //   Groups: every x block its own while there are at most 16 (128^2 x 1024, 8 / 4
-//   groups: 20.3 / 23.5 us), else a divisor of 4 to 8: the partials (1.6 MB each
+//   groups: 20.3 / 23.5 us; all with x-mode sums of one slot at a time), else a divisor of 4 to 8: the partials (1.6 MB each
 //   at 400 columns of 1024) would come near the field's own bytes.  Their memory
 //   is at most 48 MiB, or what one partial per up to 4 blocks of 16 rows takes.
 constexpr int kModeRowsPerWarp = 2;
