@@ -495,7 +495,10 @@ __device__ __forceinline__ void mirror_fetch(const V (&v)[GroupShape<L>::E], V (
 // Programmatic dependent launch of a stage after the one before it: it is set up
 // while that one's last CTAs run, reads tables, and calls wait_stage() before it
 // touches anything a kernel writes (the call returns when every kernel before
-// has completed and its writes are visible).  128^2 x 1024 launched one solve
+// has completed and its writes are visible).  What a kernel before it may have
+// written (the caller's fields too) is read by plain loads or asynchronous copies:
+// __ldg (ld.global.nc) is for memory that nothing writes while the kernel is
+// resident, which here begins before its predecessor has ended.  128^2 x 1024 launched one solve
 // after the other: 49.6 -> 45.5 us, 64^2 x 256 20.8 -> 17.0 us.  No stage lets
 // the next in before its CTAs end (griddepcontrol.launch_dependents): the next
 // one's CTAs then take the place of its own, 51.6 us.

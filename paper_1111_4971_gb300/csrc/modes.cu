@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(kBandThreads) mode_band_kernel(ModeArgs<T> a, 
     for (int e = 0; e < EV; ++e) v[e] = T(0);
 #pragma unroll 4
     for (int s = 0; s < groups; ++s) {
-      const V p = __ldg(reinterpret_cast<const V*>(a.part + (size_t(s) * a.mc + c) * a.nz) + q);
+      const V p = reinterpret_cast<const V*>(a.part + (size_t(s) * a.mc + c) * a.nz)[q];
       const T* pe = reinterpret_cast<const T*>(&p);
 #pragma unroll
       for (int e = 0; e < EV; ++e) v[e] += pe[e];

@@ -219,7 +219,7 @@ __device__ __forceinline__ unsigned absmax(unsigned m, double2 v) {
 }
 
 __device__ __forceinline__ double2 load2(const double* p, bool on) {
-  return on ? __ldg(reinterpret_cast<const double2*>(p)) : make_double2(0.0, 0.0);
+  return on ? *reinterpret_cast<const double2*>(p) : make_double2(0.0, 0.0);
 }
 
 // Tiles whose largest value is below 2^-959 are read with a factor of 2^128, so

@@ -74,7 +74,7 @@ __device__ __forceinline__ void z_scan(const ModeArgs<T>& a, int groups, int blk
       const V* src = reinterpret_cast<const V*>(a.part + (size_t(s) * a.mc + col) * NZ + t * kV);
       T g[kV];
 #pragma unroll
-      for (int i = 0; i < kV / EV; ++i) *reinterpret_cast<V*>(g + EV * i) = __ldg(src + i);
+      for (int i = 0; i < kV / EV; ++i) *reinterpret_cast<V*>(g + EV * i) = src[i];
 #pragma unroll
       for (int j = 0; j < kV; ++j) {
         const T sum = x[j] + g[j], d = sum - x[j];

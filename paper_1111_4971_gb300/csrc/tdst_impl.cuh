@@ -260,7 +260,7 @@ struct TDst {
       const int n = t + G * e;
       const int j = e < H ? 2 * n : 2 * N - 1 - 2 * n;
       const float2 f = __half22float2(row[j]);
-      const float sc = __ldg(&zs[(i * N + j) / a.zcols]) * (e < H ? 1.f : -1.f);
+      const float sc = zs[(i * N + j) / a.zcols] * (e < H ? 1.f : -1.f);
       v[e] = mk<V>(T(f.x * sc), T(f.y * sc));
     }
   }

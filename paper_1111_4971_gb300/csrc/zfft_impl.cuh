@@ -231,7 +231,7 @@ __device__ __forceinline__ void zfwd_tile(const SolveArgs<T>& a, int tile, unsig
   V v[E];
   const V* src = reinterpret_cast<const V*>(a.rho + size_t(valid ? col : 0) * NZ);
 #pragma unroll
-  for (int e = 0; e < E; ++e) v[e] = valid ? __ldg(&src[t + G * e]) : mk<V>(0, 0);
+  for (int e = 0; e < E; ++e) v[e] = valid ? src[t + G * e] : mk<V>(0, 0);
   if (p) {
     const V b = __ldg(&a.w2_z[2 * t]);
 #pragma unroll
@@ -333,11 +333,11 @@ __device__ __forceinline__ void zinv_tile(const SolveArgs<T>& a, int tile, unsig
     for (int e = 0; e < E; ++e) {
       const int k = 2 * (t + G * e) + p;
       const float2 f = __half22float2(mycol[k]);
-      const float sc = __ldg(&rs[size_t(k) * a.nx]);
+      const float sc = rs[size_t(k) * a.nx];
       v[e] = mk<V>(T(f.x * sc), T(f.y * sc));
     }
     const float2 f = __half22float2(mycol[NZ]);
-    const float sc = __ldg(&rs[size_t(NZ) * a.nx]);
+    const float sc = rs[size_t(NZ) * a.nx];
     V xN = mk<V>(T(f.x * sc), T(f.y * sc));
     __syncthreads();                                  // staging tile becomes FFT scratch
     if (CONJ) {
