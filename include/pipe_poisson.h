@@ -365,6 +365,8 @@ int pipe_mode_spectrum(pipe_handle* h, double* out, size_t count);
  *            phi[i][j][k] = sum_{m,n} sin(m pi x_i/a) sin(n pi y_j/b) psi[c][k]
  * The three in a row are the solve of this form (pipe_poisson_solve with plan
  * t_kind 3); it is symmetric, so the adjoint is the same chain.
+ * FP64: a value of stage 0's or stage 2's input that is not finite makes the
+ * outputs of its tile of 16 z planes NaN (in a solve: of its own z plane).
  * FP64 stages 0 and 2 keep the half-transformed field in the handle's
  * workspace, as a solve does: one such call or solve per handle at a time.
  * Errors: PIPE_EINVAL (stage outside 0..2, null or misaligned pointers),

@@ -290,10 +290,11 @@ ModeArgs<T> mode_args(const pipe_handle* h, const void* rho, void* phi, void* pa
   return a;
 }
 
-// one stage; `half`: FP64's buffer of the half-transformed field
+// one stage; FP64: `half` is the buffer of the half-transformed field, `nan_tile`
+// as SplitArgs
 template <typename T>
 int mode_stage(const pipe_handle* h, int stage, const void* rho, void* phi, void* part, void* psi, void* half,
-               cudaStream_t st) {
+               bool nan_tile, cudaStream_t st) {
   const ModeArgs<T> a = mode_args<T>(h, rho, phi, part, psi);
   if (stage == 1) return status_of(launch_mode_z_stage<T>(a, st));
   if constexpr (sizeof(T) == 4) {
@@ -307,6 +308,7 @@ int mode_stage(const pipe_handle* h, int stage, const void* rho, void* phi, void
     s.fold = h->fy;
     s.half = static_cast<double*>(half);
     s.zs = split_slab(a.nx, h->myp, a.nz);
+    s.nan_tile = nan_tile;
     return status_of(stage == 0 ? launch_split_project(s, a.rho, a.part, st) : launch_split_back(s, a.psi, a.phi, st));
   }
 }
@@ -321,8 +323,8 @@ int mode_solve(pipe_handle* h, const void* rho, void* phi, void* scratch, cudaSt
   char* psi = static_cast<char*>(scratch) + size_t(mode_xblocks(h)) * column;
   int s = PIPE_OK;
   for (int stage = 0; stage < 3 && s == PIPE_OK; ++stage)
-    s = h->grid.dtype == PIPE_F64 ? mode_stage<double>(h, stage, rho, phi, scratch, psi, psi + column, st)
-                                  : mode_stage<float>(h, stage, rho, phi, scratch, psi, nullptr, st);
+    s = h->grid.dtype == PIPE_F64 ? mode_stage<double>(h, stage, rho, phi, scratch, psi, psi + column, false, st)
+                                  : mode_stage<float>(h, stage, rho, phi, scratch, psi, nullptr, false, st);
   return s;
 }
 
@@ -755,10 +757,10 @@ int pipe_stage_modes(pipe_handle* h, int stage, const void* in, void* out, void*
   void* part = stage == 0 ? out : (stage == 1 ? vin : nullptr);
   void* psi = stage == 1 ? out : (stage == 2 ? vin : nullptr);
   void* phi = stage == 2 ? out : nullptr;
-  if (h->grid.dtype != PIPE_F64) return mode_stage<float>(h, stage, rho, phi, part, psi, nullptr, s);
+  if (h->grid.dtype != PIPE_F64) return mode_stage<float>(h, stage, rho, phi, part, psi, nullptr, true, s);
   // the half-transformed field is the handle's, as in a solve
   char* half = static_cast<char*>(h->mwork) + sizeof(double) * size_t(mode_xblocks(h) + 1) * h->mxp * h->myp * h->grid.nz;
-  return mode_stage<double>(h, stage, rho, phi, part, psi, half, s);
+  return mode_stage<double>(h, stage, rho, phi, part, psi, half, true, s);
 }
 
 }  // extern "C"

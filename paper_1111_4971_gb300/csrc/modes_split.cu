@@ -4,7 +4,7 @@
 // GB300's FP64 pipe does 2 FMAs per clock and SM (1.1 TFLOP/s in all), so the
 // FP64 mode sums were bound by it: 512 of 520 us of a 128^2 x 1024 projection.
 // Here every FP64 factor is split into 6 signed digits of 9 bits (54 bits
-// below the largest value of its tile; the scheme of Ozaki, Ogita, Oishi and
+// below the largest value it is summed with; the scheme of Ozaki, Ogita, Oishi and
 // Rump, "Error-free transformations of matrix multiplication by using fast
 // routines of matrix multiplication", 2012), each digit a small integer that
 // FP16 holds exactly.  Digit products are summed by FP16 MMA with FP32
@@ -28,8 +28,13 @@
 // are 8 table columns.  The table's digits come as ready fragments (three
 // 16-byte loads per lane, L1 hits shared by the CTA's warps).
 //
-// The scale of a warp's tile is the exponent of its largest value: the tile is
-// read twice, first for the maximum, then for the digits.
+// The scale is a power of two per z plane of a warp's tile, the exponent of the
+// plane's largest value over the rows: planes are independent in both sums, so a
+// plane's accuracy is its own, whatever the 15 beside it hold (one scale a tile
+// left a plane 2^k below its tile 54 - k bits).  A lane holds two planes, as rows
+// g and g + 8 of A and of the accumulators; their maxima go over the four lanes of
+// equal g by shuffles: 168.4 -> 171.6 us at 128^2 x 1024, 305.2 -> 306.0 at 256^2
+// x 512.  The tile is read twice, first for the maxima, then for the digits.
 // Splitting costs some 45 integer instructions a value and putting an output
 // together some 30; they bound the two kernels (ALU pipe 48 and 55 % busy,
 // tensor pipe 21 and 38 %, DRAM 25 and 35 %, 11 warps an SM held to that by the
@@ -39,7 +44,8 @@
 // folds too) 3230 -> 325 us.  Error against 64 bits over such meshes 4 to 8e-16,
 // the FP64 FMA sums' 4 to 9e-16.
 //
-// Values that are not finite give NaN in every output of the tile.
+// Values that are not finite give NaN in every output of their z plane (a stage
+// run by itself, pipe_stage_modes: of their 16 planes).
 #include <cuda_fp16.h>
 
 #include <cmath>
@@ -193,9 +199,9 @@ struct Exponent {
 };
 // v 2^extra (a call, so that it is branched around and not predicated: the
 // FP64 pipe would be taken all the same)
-__device__ __noinline__ double2 rescale(double2 v, int extra) {
-  const double f = extra < 0 ? 0x1p-300 : 0x1p300;
-  return make_double2(v.x * f, v.y * f);
+__device__ __noinline__ double2 rescale(double2 v, int extra0, int extra1) {
+  auto factor = [](int extra) { return extra == 0 ? 1.0 : (extra < 0 ? 0x1p-300 : 0x1p300); };
+  return make_double2(v.x * factor(extra0), v.y * factor(extra1));
 }
 template <bool CVT>
 __device__ __forceinline__ double to_double(long long v, int e) {
@@ -213,19 +219,44 @@ __device__ __forceinline__ double to_double(long long v, int e) {
   }
 }
 
-// the larger of m and the high words of v, signs off
-__device__ __forceinline__ unsigned absmax(unsigned m, double2 v) {
-  return max(m, max(unsigned(__double2hiint(v.x)) & 0x7fffffffu, unsigned(__double2hiint(v.y)) & 0x7fffffffu));
+// Per z plane of a lane (x: plane 2g, y: plane 2g + 1): the larger of m and the
+// high words of v, signs off; and the larger (the union) over the four lanes
+// that hold the plane
+__device__ __forceinline__ uint2 absmax(uint2 m, double2 v) {
+  return make_uint2(max(m.x, unsigned(__double2hiint(v.x)) & 0x7fffffffu),
+                    max(m.y, unsigned(__double2hiint(v.y)) & 0x7fffffffu));
+}
+__device__ __forceinline__ uint2 plane_max(uint2 m) {
+#pragma unroll
+  for (int d = 1; d < 4; d *= 2)
+    m = make_uint2(max(m.x, __shfl_xor_sync(0xffffffffu, m.x, d)), max(m.y, __shfl_xor_sync(0xffffffffu, m.y, d)));
+  return m;
+}
+__device__ __forceinline__ uint2 plane_or(uint2 m) {
+#pragma unroll
+  for (int d = 1; d < 4; d *= 2) {
+    m.x |= __shfl_xor_sync(0xffffffffu, m.x, d);
+    m.y |= __shfl_xor_sync(0xffffffffu, m.y, d);
+  }
+  return m;
 }
 
 __device__ __forceinline__ double2 load2(const double* p, bool on) {
   return on ? *reinterpret_cast<const double2*>(p) : make_double2(0.0, 0.0);
 }
 
-// Tiles whose largest value is below 2^-959 are read with a factor of 2^128, so
+// Planes whose largest value is below 2^-959 are read with a factor of 2^128, so
 // that to_fixed holds for them too.
 constexpr int kTiny = 64;
-__device__ __forceinline__ double2 raise(double2 v) { return make_double2(v.x * 0x1p128, v.y * 0x1p128); }
+__device__ __forceinline__ double2 raise(double2 v, bool x, bool y) {
+  return make_double2(x ? v.x * 0x1p128 : v.x, y ? v.y * 0x1p128 : v.y);
+}
+// NaN for a plane whose largest value is not finite
+constexpr unsigned kNotFinite = 0x7ff00000u;
+__device__ __forceinline__ double2 nan_where(double2 v, int emax0, int emax1) {
+  const double nan = __longlong_as_double(0x7ff8000000000000LL);
+  return make_double2(emax0 == 0x7ff ? nan : v.x, emax1 == 0x7ff ? nan : v.y);
+}
 
 // Contraction.  NT column tiles (FOLD: the first NT / 2 take the sums of the
 // mirror pairs, the others their differences).
@@ -239,6 +270,7 @@ struct ContractArgs {
   int rows;                  // output rows (slots)
   int mirror;                // FOLD: row k's mirror is row mirror - k
   int wall;                  // FOLD: pair 0 is row 0 (on the wall, table zero) and row `wall`
+  int nan_tile;              // a value that is not finite takes the 16 planes of its tile, not its own alone
 };
 
 // A warp's tile in shared memory: [k step of the run][row, mirror row][16 rows][16 z],
@@ -301,39 +333,44 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 3) split_contract_kernel(con
     const int n1 = unit2 < units ? min(n0 + kSeg / 16, steps) : n0;
     cp_async_wait<0>();
     __syncwarp();
-    unsigned m = 0;
+    uint2 m = make_uint2(0, 0);
 #pragma unroll 1
     for (int ks = s0; ks < s1; ++ks)
 #pragma unroll
       for (int i = 0; i < (FOLD ? 8 : 4); ++i) m = absmax(m, value(ks, i >> 2, i & 3));
-    m = __reduce_max_sync(0xffffffffu, m);
-    const bool bad = m >= 0x7ff00000u;
-    bool tiny = false;
-    if (m == 0) {                                      // zeros, but for values below 2^-1042
+    m = plane_max(m);
+    if (a.nan_tile && __any_sync(0xffffffffu, max(m.x, m.y) >= kNotFinite)) m = make_uint2(kNotFinite, kNotFinite);
+    bool tiny0 = false, tiny1 = false;
+    constexpr unsigned kLow = unsigned(kTiny) << 20;
+    if (__any_sync(0xffffffffu, min(m.x, m.y) < kLow)) {
+      // planes of zeros, common outside a bunch, or without a value of 2^-959 or more
+      uint2 any = make_uint2(0, 0);
 #pragma unroll 1
       for (int ks = s0; ks < s1; ++ks)
 #pragma unroll
         for (int i = 0; i < (FOLD ? 8 : 4); ++i) {
           const double2 v = value(ks, i >> 2, i & 3);
-          m |= unsigned(__double2loint(v.x)) | unsigned(__double2loint(v.y));
+          any.x |= unsigned(__double2hiint(v.x)) << 1 | unsigned(__double2loint(v.x));
+          any.y |= unsigned(__double2hiint(v.y)) << 1 | unsigned(__double2loint(v.y));
         }
-      m = __reduce_or_sync(0xffffffffu, m) != 0;
-    }
-    if (m != 0 && m < unsigned(kTiny) << 20) {         // no value of 2^-959 or more
-      m = 0;
+      any = plane_or(any);
+      tiny0 = m.x < kLow && any.x != 0;
+      tiny1 = m.y < kLow && any.y != 0;
+      if (__any_sync(0xffffffffu, tiny0 || tiny1)) {
+        uint2 r = make_uint2(0, 0);
 #pragma unroll 1
-      for (int ks = s0; ks < s1; ++ks)
+        for (int ks = s0; ks < s1; ++ks)
 #pragma unroll 1
-        for (int i = 0; i < (FOLD ? 8 : 4); ++i) {
-          const double2 v = raise(value(ks, i >> 2, i & 3));
-          m = absmax(m, v);
-          if (16 * ks + 8 * ((i & 3) >> 1) < a.K) *slot(ks, i >> 2, i & 3) = v;
-        }
-      m = __reduce_max_sync(0xffffffffu, m);
-      tiny = true;
+          for (int i = 0; i < (FOLD ? 8 : 4); ++i) {
+            const double2 v = raise(value(ks, i >> 2, i & 3), tiny0, tiny1);
+            r = absmax(r, v);
+            if (16 * ks + 8 * ((i & 3) >> 1) < a.K) *slot(ks, i >> 2, i & 3) = v;
+          }
+        m = plane_max(r);
+      }
     }
-    const bool zero = m == 0;                          // nothing there: common outside a bunch
-    const int emax = max(int(m >> 20), kTiny);
+    const bool zero = !__any_sync(0xffffffffu, (m.x | m.y) != 0);   // nothing there
+    const int emax0 = max(int(m.x >> 20), kTiny), emax1 = max(int(m.y >> 20), kTiny);   // 0x7ff: not finite
     float acc[NT][kD][4];
 #pragma unroll
     for (int n = 0; n < NT; ++n)
@@ -367,13 +404,13 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 3) split_contract_kernel(con
         if constexpr (FOLD) {
           if (i == 0 && a.wall && ks == 0 && t == 0) u = make_double2(0.0, 0.0);
           const double2 v = value(ks, 1, i);
-          const Fixed u0 = to_fixed(u.x, emax), v0 = to_fixed(v.x, emax);
-          const Fixed u1 = to_fixed(u.y, emax), v1 = to_fixed(v.y, emax);
+          const Fixed u0 = to_fixed(u.x, emax0), v0 = to_fixed(v.x, emax0);
+          const Fixed u1 = to_fixed(u.y, emax1), v1 = to_fixed(v.y, emax1);
           P[i][0] = fixed_sum(u0, v0); Q[i][0] = fixed_difference(u0, v0);
           P[i][1] = fixed_sum(u1, v1); Q[i][1] = fixed_difference(u1, v1);
         } else {
-          P[i][0] = fixed_value(to_fixed(u.x, emax));
-          P[i][1] = fixed_value(to_fixed(u.y, emax));
+          P[i][0] = fixed_value(to_fixed(u.x, emax0));
+          P[i][1] = fixed_value(to_fixed(u.y, emax1));
         }
       }
       __syncwarp();                                    // every lane has this step's values
@@ -390,7 +427,7 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 3) split_contract_kernel(con
 #pragma unroll 1
     for (int ks = n0 + s1 - s0; ks < n1; ++ks) copy(unit2, ks);     // a longer run follows
     // V 2^-8 = acc_0 2^37 + acc_1 2^28 + acc_2 2^19 + (acc_3 2^18 + acc_4 2^9 + acc_5) 2^-8
-    const Exponent e(emax - 1075 - (tiny ? 128 : 0));
+    const Exponent e0(emax0 - 1075 - (tiny0 ? 128 : 0)), e1(emax1 - 1075 - (tiny1 ? 128 : 0));
     const int o = unit / a.ztiles;
     double* out = a.out + size_t(o) * a.out_o + (unit - o * a.ztiles) * 16 + 2 * g;
 #pragma unroll
@@ -409,9 +446,9 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 3) split_contract_kernel(con
         if (q < (FOLD ? half : a.rows)) {
           double2* p = reinterpret_cast<double2*>(out + size_t(r) * a.out_r);
           double2 w = make_double2(0.0, 0.0);
-          if (!zero) w = make_double2(to_double<false>(fixed(c), e.e), to_double<true>(fixed(2 + c), e.e));
-          if (e.extra) w = rescale(w, e.extra);
-          if (bad) w = make_double2(__longlong_as_double(0x7ff8000000000000LL), __longlong_as_double(0x7ff8000000000000LL));
+          if (!zero) w = make_double2(to_double<false>(fixed(c), e0.e), to_double<true>(fixed(2 + c), e1.e));
+          if (e0.extra | e1.extra) w = rescale(w, e0.extra, e1.extra);
+          w = nan_where(w, emax0, emax1);
           if (s0 > 0) {
             const double2 b = *p;
             w.x += b.x;
@@ -441,6 +478,7 @@ struct ExpandArgs {
   int K;                     // modes (FOLD: both halves)
   int tiles;                 // output rows / 8 (FOLD: pairs / 8)
   int mirror, wall;          // as ContractArgs
+  int nan_tile;
 };
 constexpr int kExtra = 2;    // |values| < 2^(53 + kExtra), |d_0| <= 256 << kExtra
 
@@ -473,12 +511,12 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 3) split_expand_kernel(const
   wait_stage();
   double2 x[KS][4];
   auto largest = [&]() {
-    unsigned m = 0;
+    uint2 m = make_uint2(0, 0);
 #pragma unroll
     for (int ks = 0; ks < KS; ++ks)
 #pragma unroll
       for (int i = 0; i < 4; ++i) m = absmax(m, x[ks][i]);
-    return __reduce_max_sync(0xffffffffu, m);
+    return plane_max(m);
   };
 #pragma unroll
   for (int ks = 0; ks < KS; ++ks)
@@ -487,16 +525,17 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 3) split_expand_kernel(const
       const int k = 16 * (ks % KH) + 2 * t + (i & 1) + 8 * (i >> 1);
       x[ks][i] = load2(in + size_t((ks / KH) * kmax + k) * a.in_k, k < kmax);
     }
-  unsigned top = largest();
-  const bool bad = top >= 0x7ff00000u, tiny = top < unsigned(kTiny) << 20;
-  if (tiny) {
+  uint2 top = largest();
+  if (a.nan_tile && __any_sync(0xffffffffu, max(top.x, top.y) >= kNotFinite)) top = make_uint2(kNotFinite, kNotFinite);
+  const bool tiny0 = top.x < unsigned(kTiny) << 20, tiny1 = top.y < unsigned(kTiny) << 20;
+  if (__any_sync(0xffffffffu, tiny0 || tiny1)) {
 #pragma unroll
     for (int ks = 0; ks < KS; ++ks)
 #pragma unroll
-      for (int i = 0; i < 4; ++i) x[ks][i] = raise(x[ks][i]);
+      for (int i = 0; i < 4; ++i) x[ks][i] = raise(x[ks][i], tiny0, tiny1);
     top = largest();
   }
-  const int emax = max(int(top >> 20), kTiny);
+  const int emax0 = max(int(top.x >> 20), kTiny), emax1 = max(int(top.y >> 20), kTiny);
   unsigned A[KS][kD][4];
 #pragma unroll
   for (int ks = 0; ks < KS; ++ks)
@@ -504,15 +543,14 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 3) split_expand_kernel(const
     for (int h = 0; h < 2; ++h) {
       const double2 u = x[ks][2 * h], v = x[ks][2 * h + 1];
       unsigned d[kD];
-      digits_round(to_fixed_round(u.x, emax), to_fixed_round(v.x, emax), d);
+      digits_round(to_fixed_round(u.x, emax0), to_fixed_round(v.x, emax0), d);
 #pragma unroll
       for (int i = 0; i < kD; ++i) A[ks][i][2 * h] = d[i];
-      digits_round(to_fixed_round(u.y, emax), to_fixed_round(v.y, emax), d);
+      digits_round(to_fixed_round(u.y, emax1), to_fixed_round(v.y, emax1), d);
 #pragma unroll
       for (int i = 0; i < kD; ++i) A[ks][i][2 * h + 1] = d[i];
     }
-  const Exponent e(emax - 1083 - kExtra + 6 - (tiny ? 128 : 0));
-  const double nan = __longlong_as_double(0x7ff8000000000000LL);
+  const Exponent e0(emax0 - 1083 - kExtra + 6 - (tiny0 ? 128 : 0)), e1(emax1 - 1083 - kExtra + 6 - (tiny1 ? 128 : 0));
   // V 2^-6 = acc_0 2^39 + acc_1 2^30 + acc_2 2^21 + acc_3 2^12 + acc_4 2^3 + acc_5 2^-6,
   // without kOff where the sums are read off with their offset M
   constexpr unsigned M = 0x4B400000u;                // the bits of 1.5 2^23
@@ -550,26 +588,26 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 3) split_expand_kernel(const
       const int r = 8 * tile + 2 * t + c;
       const unsigned long long o0 = fixed(acc[0], c), o1 = fixed(acc[0], 2 + c);
       if constexpr (FOLD) {
-        const unsigned long long e0 = fixed(acc[1], c), e1 = fixed(acc[1], 2 + c);
-        double2 lo = make_double2(to_double<false>(static_cast<long long>(o0 + e0 - 2 * kOff), e.e),
-                                  to_double<false>(static_cast<long long>(o1 + e1 - 2 * kOff), e.e));
-        double2 hi = make_double2(to_double<true>(static_cast<long long>(o0 - e0), e.e),
-                                  to_double<true>(static_cast<long long>(o1 - e1), e.e));
-        if (e.extra) {
-          lo = rescale(lo, e.extra);
-          hi = rescale(hi, e.extra);
+        const unsigned long long v0 = fixed(acc[1], c), v1 = fixed(acc[1], 2 + c);
+        double2 lo = make_double2(to_double<false>(static_cast<long long>(o0 + v0 - 2 * kOff), e0.e),
+                                  to_double<false>(static_cast<long long>(o1 + v1 - 2 * kOff), e1.e));
+        double2 hi = make_double2(to_double<true>(static_cast<long long>(o0 - v0), e0.e),
+                                  to_double<true>(static_cast<long long>(o1 - v1), e1.e));
+        if (e0.extra | e1.extra) {
+          lo = rescale(lo, e0.extra, e1.extra);
+          hi = rescale(hi, e0.extra, e1.extra);
         }
         const bool on_wall = a.wall && r == 0;
         if (on_wall) lo = make_double2(0.0, 0.0);
-        if (bad) lo = hi = make_double2(nan, nan);
+        lo = nan_where(lo, emax0, emax1);
+        hi = nan_where(hi, emax0, emax1);
         *reinterpret_cast<double2*>(out + size_t(r) * a.out_r) = lo;
         *reinterpret_cast<double2*>(out + size_t(on_wall ? a.wall : a.mirror - r) * a.out_r) = hi;
       } else {
-        double2 v = make_double2(to_double<false>(static_cast<long long>(o0 - kOff), e.e),
-                                 to_double<true>(static_cast<long long>(o1 - kOff), e.e));
-        if (e.extra) v = rescale(v, e.extra);
-        if (bad) v = make_double2(nan, nan);
-        *reinterpret_cast<double2*>(out + size_t(r) * a.out_r) = v;
+        double2 v = make_double2(to_double<false>(static_cast<long long>(o0 - kOff), e0.e),
+                                 to_double<true>(static_cast<long long>(o1 - kOff), e1.e));
+        if (e0.extra | e1.extra) v = rescale(v, e0.extra, e1.extra);
+        *reinterpret_cast<double2*>(out + size_t(r) * a.out_r) = nan_where(v, emax0, emax1);
       }
     }
   }
@@ -716,6 +754,7 @@ cudaError_t launch_split_project(const SplitArgs& s, const double* rho, double* 
     y.rows = s.myp;
     y.mirror = s.fold == 2 ? s.ny : s.ny - 1;
     y.wall = s.fold == 2 ? s.ny / 2 : 0;
+    y.nan_tile = s.nan_tile;
     cudaError_t e = contract(y, fold, st);
     if (e != cudaSuccess) return e;
     ContractArgs x{};
@@ -730,6 +769,7 @@ cudaError_t launch_split_project(const SplitArgs& s, const double* rho, double* 
     x.ztiles = s.zs / 16;
     x.K = s.nx;
     x.rows = s.mxp;
+    x.nan_tile = s.nan_tile;
     if ((e = contract(x, false, st)) != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -750,6 +790,7 @@ cudaError_t launch_split_back(const SplitArgs& s, const double* psi, double* phi
     x.ztiles = s.zs / 16;
     x.K = s.mxp;
     x.tiles = s.nx / 8;
+    x.nan_tile = s.nan_tile;
     cudaError_t e = expand(x, false, s.ex_small, st);
     if (e != cudaSuccess) return e;
     ExpandArgs y{};
@@ -766,6 +807,7 @@ cudaError_t launch_split_back(const SplitArgs& s, const double* psi, double* phi
     y.tiles = (fold ? s.ny / 2 : s.ny) / 8;
     y.mirror = s.fold == 2 ? s.ny : s.ny - 1;
     y.wall = s.fold == 2 ? s.ny / 2 : 0;
+    y.nan_tile = s.nan_tile;
     if ((e = expand(y, fold, s.ey_small, st)) != cudaSuccess) return e;
   }
   return cudaSuccess;

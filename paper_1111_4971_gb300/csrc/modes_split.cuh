@@ -45,6 +45,7 @@ struct SplitArgs {
   int fold;                  // 0: all rows, 1: mirror pairs (j, ny-1-j), 2: (j, ny-j) with row 0 on the wall
   double* half;
   int zs;
+  int nan_tile;              // 1: a value that is not finite makes its 16 planes' outputs NaN (single stages), 0: its own plane's
 };
 // z values per slab: the half-transformed field of a slab is at most 32 MiB
 // (it stays in L2 between the kernel that writes it and the one that reads it)
