@@ -302,6 +302,7 @@ int mode_stage(const pipe_handle* h, int stage, const void* rho, void* phi, void
   } else {
     SplitArgs s{};
     s.cy = h->mcy; s.cx = h->mcx; s.ey = h->mey; s.ex = h->mex;
+    s.ys = h->mys; s.xs = h->mxs;
     s.ey_small = h->mey_small; s.ex_small = h->mex_small;
     s.nx = a.nx; s.ny = a.ny; s.nz = a.nz;
     s.mx = a.mx; s.mxp = h->mxp; s.myp = h->myp;
@@ -483,29 +484,46 @@ static int setup_pipe(const pipe_geometry* geom, const pipe_grid* grid, int igf,
       const bool halves = h->fy != 0;
       const size_t n[4] = {split_contract_size(nyk, h->myp, halves), split_contract_size(grid->nx, h->mxp, false),
                            split_expand_size(nyk, h->myp, halves), split_expand_size(grid->nx, h->mxp, false)};
-      if (cudaMalloc(&h->msplit, (n[0] + n[1] + n[2] + n[3]) * sizeof(uint4)) != cudaSuccess) {
+      const int npy = split_padded(nyk), npx = split_padded(grid->nx);       // multiples of 16
+      if (cudaMalloc(&h->msplit, (n[0] + n[1] + n[2] + n[3]) * sizeof(uint4) + size_t(npy + npx) * sizeof(int)) !=
+          cudaSuccess) {
         free_handle(h);
         return PIPE_ENOMEM;
       }
       h->mcy = h->msplit; h->mcx = h->mcy + n[0]; h->mey = h->mcx + n[1]; h->mex = h->mey + n[2];
-      if ((e = build_split_table(h->msy64, nyk, h->myp, halves, false, h->mcy, nullptr)) != cudaSuccess ||
-          (e = build_split_table(h->msx64, grid->nx, h->mxp, false, false, h->mcx, nullptr)) != cudaSuccess ||
-          (e = build_split_table(h->msy64, nyk, h->myp, halves, true, h->mey, nullptr)) != cudaSuccess ||
-          (e = build_split_table(h->msx64, grid->nx, h->mxp, false, true, h->mex, nullptr)) != cudaSuccess ||
+      int* rows = reinterpret_cast<int*>(h->mex + n[3]);
+      double* t = static_cast<double*>(std::malloc((nsx > nsy ? nsx : nsy) * sizeof(double)));
+      int* scale = static_cast<int*>(std::malloc(size_t(npy + npx) * sizeof(int)));
+      if (!t || !scale) {
+        std::free(t);
+        std::free(scale);
+        free_handle(h);
+        return PIPE_ENOMEM;
+      }
+      e = cudaMemcpy(t, h->msy64, nsy * sizeof(double), cudaMemcpyDeviceToHost);
+      if (e == cudaSuccess) {
+        h->mys = table_scales(t, nyk, h->myp, scale);
+        h->mey_small = expand_sums_small(t, scale, nyk, h->myp, halves);
+        e = cudaMemcpy(t, h->msx64, nsx * sizeof(double), cudaMemcpyDeviceToHost);
+      }
+      if (e == cudaSuccess) {
+        h->mxs = table_scales(t, grid->nx, h->mxp, scale + npy);
+        h->mex_small = expand_sums_small(t, scale + npy, grid->nx, h->mxp, false);
+        e = cudaMemcpy(rows, scale, size_t(npy + npx) * sizeof(int), cudaMemcpyHostToDevice);
+      }
+      h->mys.rows = rows;
+      h->mxs.rows = rows + npy;
+      std::free(t);
+      std::free(scale);
+      if (e != cudaSuccess ||
+          (e = build_split_table(h->msy64, h->mys.rows, nyk, h->myp, halves, false, h->mcy, nullptr)) != cudaSuccess ||
+          (e = build_split_table(h->msx64, h->mxs.rows, grid->nx, h->mxp, false, false, h->mcx, nullptr)) != cudaSuccess ||
+          (e = build_split_table(h->msy64, h->mys.rows, nyk, h->myp, halves, true, h->mey, nullptr)) != cudaSuccess ||
+          (e = build_split_table(h->msx64, h->mxs.rows, grid->nx, h->mxp, false, true, h->mex, nullptr)) != cudaSuccess ||
           (e = cudaStreamSynchronize(nullptr)) != cudaSuccess) {
         free_handle(h);
         return status_of(e);
       }
-      double* t = static_cast<double*>(std::malloc((nsx > nsy ? nsx : nsy) * sizeof(double)));
-      if (!t) { free_handle(h); return PIPE_ENOMEM; }
-      e = cudaMemcpy(t, h->msy64, nsy * sizeof(double), cudaMemcpyDeviceToHost);
-      if (e == cudaSuccess) {
-        h->mey_small = expand_sums_small(t, nyk, h->myp, halves);
-        e = cudaMemcpy(t, h->msx64, nsx * sizeof(double), cudaMemcpyDeviceToHost);
-      }
-      if (e == cudaSuccess) h->mex_small = expand_sums_small(t, grid->nx, h->mxp, false);
-      std::free(t);
-      if (e != cudaSuccess) { free_handle(h); return status_of(e); }
     }
     if (n_nb >= 0) {                     // the banded operator's z stencil
       const size_t nkb = size_t(h->mxp) * h->myp * (n_nb + 1);

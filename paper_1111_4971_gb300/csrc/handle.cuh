@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/pipe_poisson.h"
+#include "modes_split.cuh"
 
 namespace pp {
 // Kernel variant choices for one handle (filled by default_plan, refined by
@@ -67,6 +68,7 @@ struct pipe_handle {
   // FP64: fragment tables of the split products (modes_split.cu), one allocation
   uint4* msplit = nullptr;
   uint4 *mcy = nullptr, *mcx = nullptr, *mey = nullptr, *mex = nullptr;
+  pp::RowScale mys{}, mxs{};                   // the tables' row scales (in the same allocation)
   bool mey_small = false, mex_small = false;   // expand_sums_small of mey, mex
   // part [groups][mc][nz], then psi [mc][nz], of the dtype; FP64: then the
   // half-transformed field of a slab (modes_split.cuh)

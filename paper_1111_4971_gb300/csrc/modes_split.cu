@@ -33,8 +33,18 @@
 // plane's accuracy is its own, whatever the 15 beside it hold (one scale a tile
 // left a plane 2^k below its tile 54 - k bits).  A lane holds two planes, as rows
 // g and g + 8 of A and of the accumulators; their maxima go over the four lanes of
-// equal g by shuffles: 168.4 -> 171.6 us at 128^2 x 1024, 305.2 -> 306.0 at 256^2
-// x 512.  The tile is read twice, first for the maxima, then for the digits.
+// equal g by shuffles.  The tile is read twice, first for the maxima, then for the
+// digits.
+// A table row has a power of two of its own too (table_scales): next to a wall
+// every sine of a row is small, and digits of the sines themselves would cut them
+// 2^-54 below 1, not below the row (100 u of the row's terms where its largest
+// sine is 0.005).  The expansion takes it off its output's exponent, the
+// contraction off the value's; a row that is zero, on the wall, takes no part in
+// the maxima.  Both together against one scale a tile: projection and
+// back-projection at 128^2 x 1024 90.5 + 70.9 -> 88.1 + 71.5 us, 256^2 x 512 on the
+// wall 190 + 128 -> 183 + 129, 48 x 80 x 512 21.4 + 18.4 -> 21.2 + 19.1: branches on
+// a plane's exponent go by a vote, and the warp's index is broadcast, so that what
+// follows from them stays in uniform registers (without: 105 us for the first).
 // Splitting costs some 45 integer instructions a value and putting an output
 // together some 30; they bound the two kernels (ALU pipe 48 and 55 % busy,
 // tensor pipe 21 and 38 %, DRAM 25 and 35 %, 11 warps an SM held to that by the
@@ -48,6 +58,7 @@
 // run by itself, pipe_stage_modes: of their 16 planes).
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <utility>
 
@@ -77,16 +88,16 @@ __device__ __forceinline__ unsigned long long pack64(unsigned hi, unsigned lo) {
   return (static_cast<unsigned long long>(hi) << 32) | lo;
 }
 
-// magnitude and sign (0 or -1) of x 2^(1075 + kGuard - emax), cut to an integer
-// below 2^(53 + kGuard); the exponent field of x is at most emax, emax >= 64 (zeros and
-// subnormal values are then shifted out)
+// magnitude and sign (0 or -1) of x 2^(1075 + kGuard - e), cut to an integer
+// below 2^(53 + kGuard); top = e 2^20; the exponent field of x is at most e, e >= 64
+// (zeros and subnormal values are then shifted out)
 struct Fixed {
   unsigned long long v;      // magnitude XOR sign
   int s;
 };
-__device__ __forceinline__ Fixed to_fixed(double x, int emax) {
+__device__ __forceinline__ Fixed to_fixed(double x, unsigned top) {
   const int hi = __double2hiint(x);
-  const unsigned sh = min(unsigned(emax - int((unsigned(hi) >> 20) & 0x7ffu)), 63u);
+  const unsigned sh = min((top - (unsigned(hi) & 0x7ff00000u)) >> 20, 63u);
   const unsigned long long m = (pack64((unsigned(hi) & 0xfffffu) | 0x100000u, unsigned(__double2loint(x))) << kGuard) >> sh;
   const int s = hi >> 31;
   return {m ^ static_cast<unsigned long long>(static_cast<long long>(s)), s};
@@ -188,33 +199,37 @@ __device__ __forceinline__ long long mad_wide_s(int a, int b, long long c) {
 // subnormal or overflows): by integer arithmetic (halves away from zero), or,
 // CVT, by the conversion instruction, which runs at 2 lanes a clock and SM: a
 // kernel gives half of its outputs to each.  Other exponents: Exponent's e,
-// then a factor of 2^300 or 2^-300.
+// then a factor of 2^300 or 2^-300 (e may then still lose a table row's scale).
 struct Exponent {
-  int e, extra;
-  __device__ __forceinline__ explicit Exponent(int x) : e(x), extra(0) {
-    if (x <= -1000) extra = -300;
-    if (x >= 900) extra = 300;
-    e -= extra;
+  int e20, extra;            // e 2^20; for values that are not finite, extra is kNan
+  static constexpr int kNan = 1;
+  __device__ __forceinline__ Exponent(int x, bool finite) : extra(0) {
+    if (x <= kMaxRowScale - 1000) extra = -300;
+    if (x >= 900) extra = finite ? 300 : kNan;
+    e20 = (x - extra) * (1 << 20);
   }
 };
-// v 2^extra (a call, so that it is branched around and not predicated: the
+// v 2^extra, or NaN (a call, so that it is branched around and not predicated: the
 // FP64 pipe would be taken all the same)
 __device__ __noinline__ double2 rescale(double2 v, int extra0, int extra1) {
-  auto factor = [](int extra) { return extra == 0 ? 1.0 : (extra < 0 ? 0x1p-300 : 0x1p300); };
+  auto factor = [](int extra) {
+    if (extra == Exponent::kNan) return __longlong_as_double(0x7ff8000000000000LL);
+    return extra == 0 ? 1.0 : (extra < 0 ? 0x1p-300 : 0x1p300);
+  };
   return make_double2(v.x * factor(extra0), v.y * factor(extra1));
 }
 template <bool CVT>
-__device__ __forceinline__ double to_double(long long v, int e) {
+__device__ __forceinline__ double to_double(long long v, int e20) {
   if constexpr (CVT) {
     const double d = __ll2double_rn(v);
     const int h = __double2hiint(d);
-    return __hiloint2double(h != 0 ? h + e * (1 << 20) : 0, __double2loint(d));
+    return __hiloint2double(h != 0 ? h + e20 : 0, __double2loint(d));
   } else {
     const int s = int(v >> 63);
     const unsigned long long u = static_cast<unsigned long long>((v ^ s) - s);
     const int lz = __clzll(static_cast<long long>(u));               // >= 1; 64 for zero
     const unsigned long long r = ((u << (lz - 1)) + 0x200u) >> 10;   // 53 bits, the first is the implicit one
-    const unsigned h = (hi32(r) + (unsigned(1085 + e - lz) << 20)) | (unsigned(s) & 0x80000000u);
+    const unsigned h = (hi32(r) + unsigned(e20) + (unsigned(1085 - lz) << 20)) | (unsigned(s) & 0x80000000u);
     return __hiloint2double(lz == 64 ? 0 : int(h), int(unsigned(r)));
   }
 }
@@ -251,12 +266,10 @@ constexpr int kTiny = 64;
 __device__ __forceinline__ double2 raise(double2 v, bool x, bool y) {
   return make_double2(x ? v.x * 0x1p128 : v.x, y ? v.y * 0x1p128 : v.y);
 }
-// NaN for a plane whose largest value is not finite
 constexpr unsigned kNotFinite = 0x7ff00000u;
-__device__ __forceinline__ double2 nan_where(double2 v, int emax0, int emax1) {
-  const double nan = __longlong_as_double(0x7ff8000000000000LL);
-  return make_double2(emax0 == 0x7ff ? nan : v.x, emax1 == 0x7ff ? nan : v.y);
-}
+// the exponent field that a plane is scaled by (0x7ff: not finite); planes of zeros
+// take any that needs no rescaling
+__device__ __forceinline__ int exponent_of(unsigned m) { return m == 0 ? 1075 : max(int(m >> 20), kTiny); }
 
 // Contraction.  NT column tiles (FOLD: the first NT / 2 take the sums of the
 // mirror pairs, the others their differences).
@@ -264,6 +277,7 @@ struct ContractArgs {
   const double* in;          // value (o, k, z) at o * in_o + k * in_k + z
   double* out;               // value (o, r, z) at o * out_o + r * out_r + z
   const uint4* tab;
+  RowScale scale;            // of the rows k
   size_t in_o, in_k, out_o, out_r;
   int outer, ztiles;         // units: outer x ztiles, 16 z each
   int K;                     // rows, or mirror pairs
@@ -305,7 +319,8 @@ __device__ __forceinline__ void copy_step(const ContractArgs& a, int unit, int k
 template <int NT, bool FOLD>
 __global__ void __launch_bounds__(32 * kSplitWarps, 3) split_contract_kernel(const __grid_constant__ ContractArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x) >> 5, 0);     // (uniform registers for what follows from it)
   const int units = a.outer * a.ztiles, stride = int(gridDim.x) * kSplitWarps;
   unsigned char* tile = smem_raw + warp * tile_bytes<FOLD>();
   constexpr int SB = (FOLD ? 2 : 1) * kStepBytes;      // bytes of a k step
@@ -321,6 +336,11 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 3) split_contract_kernel(con
   auto value = [&](int ks, int half, int i) __attribute__((always_inline)) {
     return 16 * ks + 8 * (i >> 1) < a.K ? *slot(ks, half, i) : make_double2(0.0, 0.0);
   };
+  // the scales of this lane's rows of a step, none in plain steps
+  auto plain = [&](int ks) __attribute__((always_inline)) { return ks >= a.scale.plain0 && ks < a.scale.plain1; };
+  auto row_scales = [&](int ks) __attribute__((always_inline)) {
+    return __ldg(reinterpret_cast<const int4*>(a.scale.rows + 16 * ks + 4 * t));
+  };
   int unit = int(blockIdx.x) * kSplitWarps + warp, s0 = 0;
   wait_stage();
   if (unit < units)
@@ -333,44 +353,68 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 3) split_contract_kernel(con
     const int n1 = unit2 < units ? min(n0 + kSeg / 16, steps) : n0;
     cp_async_wait<0>();
     __syncwarp();
-    uint2 m = make_uint2(0, 0);
+    // per plane, the largest high word of the values, each less its row's scale (a
+    // table row that is zero takes no part, nor does the row on the wall)
+    uint2 raw0 = make_uint2(0, 0);
+    if (FOLD && a.wall && s0 == 0 && t == 0) {
+      raw0 = absmax(raw0, *slot(0, 0, 0));
+      *slot(0, 0, 0) = make_double2(0.0, 0.0);
+    }
+    uint2 low;                                         // the low words of all values together
+    auto largest = [&]() __attribute__((always_inline)) {
+      uint2 m = make_uint2(0, 0), raw = raw0;
+      low = make_uint2(0, 0);
 #pragma unroll 1
-    for (int ks = s0; ks < s1; ++ks)
+      for (int ks = s0; ks < s1; ++ks) {
+        if (plain(ks)) {
 #pragma unroll
-      for (int i = 0; i < (FOLD ? 8 : 4); ++i) m = absmax(m, value(ks, i >> 2, i & 3));
-    m = plane_max(m);
+          for (int i = 0; i < (FOLD ? 8 : 4); ++i) {
+            const double2 v = value(ks, i >> 2, i & 3);
+            m = absmax(m, v);
+            low = make_uint2(low.x | unsigned(__double2loint(v.x)), low.y | unsigned(__double2loint(v.y)));
+          }
+        } else {
+          const int4 cs = row_scales(ks);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            uint2 h = make_uint2(0, 0);
+#pragma unroll
+            for (int half = 0; half < (FOLD ? 2 : 1); ++half) {
+              const double2 v = value(ks, half, i);
+              h = absmax(h, v);
+              low = make_uint2(low.x | unsigned(__double2loint(v.x)), low.y | unsigned(__double2loint(v.y)));
+            }
+            const int c = i < 2 ? (i == 0 ? cs.x : cs.y) : (i == 2 ? cs.z : cs.w);
+            raw = make_uint2(max(raw.x, h.x), max(raw.y, h.y));
+            m = make_uint2(unsigned(max(int(m.x), int(h.x) - c)), unsigned(max(int(m.y), int(h.y) - c)));
+          }
+        }
+      }
+      low = make_uint2(low.x | raw.x, low.y | raw.y);
+      return plane_max(make_uint2(raw.x >= kNotFinite ? raw.x : m.x, raw.y >= kNotFinite ? raw.y : m.y));
+    };
+    uint2 m = largest();
     if (a.nan_tile && __any_sync(0xffffffffu, max(m.x, m.y) >= kNotFinite)) m = make_uint2(kNotFinite, kNotFinite);
-    bool tiny0 = false, tiny1 = false;
+    bool tiny0 = false, tiny1 = false, zero = false;
     constexpr unsigned kLow = unsigned(kTiny) << 20;
     if (__any_sync(0xffffffffu, min(m.x, m.y) < kLow)) {
       // planes of zeros, common outside a bunch, or without a value of 2^-959 or more
-      uint2 any = make_uint2(0, 0);
-#pragma unroll 1
-      for (int ks = s0; ks < s1; ++ks)
-#pragma unroll
-        for (int i = 0; i < (FOLD ? 8 : 4); ++i) {
-          const double2 v = value(ks, i >> 2, i & 3);
-          any.x |= unsigned(__double2hiint(v.x)) << 1 | unsigned(__double2loint(v.x));
-          any.y |= unsigned(__double2hiint(v.y)) << 1 | unsigned(__double2loint(v.y));
-        }
-      any = plane_or(any);
+      const uint2 any = plane_or(make_uint2(low.x | m.x, low.y | m.y));
       tiny0 = m.x < kLow && any.x != 0;
       tiny1 = m.y < kLow && any.y != 0;
       if (__any_sync(0xffffffffu, tiny0 || tiny1)) {
-        uint2 r = make_uint2(0, 0);
 #pragma unroll 1
         for (int ks = s0; ks < s1; ++ks)
 #pragma unroll 1
-          for (int i = 0; i < (FOLD ? 8 : 4); ++i) {
-            const double2 v = raise(value(ks, i >> 2, i & 3), tiny0, tiny1);
-            r = absmax(r, v);
-            if (16 * ks + 8 * ((i & 3) >> 1) < a.K) *slot(ks, i >> 2, i & 3) = v;
-          }
-        m = plane_max(r);
+          for (int i = 0; i < (FOLD ? 8 : 4); ++i)
+            if (16 * ks + 8 * ((i & 3) >> 1) < a.K)
+              *slot(ks, i >> 2, i & 3) = raise(value(ks, i >> 2, i & 3), tiny0, tiny1);
+        m = largest();
       }
+      zero = !__any_sync(0xffffffffu, (m.x | m.y) != 0);
     }
-    const bool zero = !__any_sync(0xffffffffu, (m.x | m.y) != 0);   // nothing there
-    const int emax0 = max(int(m.x >> 20), kTiny), emax1 = max(int(m.y >> 20), kTiny);   // 0x7ff: not finite
+    const int emax0 = exponent_of(m.x), emax1 = exponent_of(m.y);
+    const unsigned top0 = unsigned(emax0) << 20, top1 = unsigned(emax1) << 20;
     float acc[NT][kD][4];
 #pragma unroll
     for (int n = 0; n < NT; ++n)
@@ -398,19 +442,21 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 3) split_contract_kernel(con
           }
       };
       unsigned long long P[4][2], Q[4][2];
+      int4 cs = make_int4(0, 0, 0, 0);
+      if (!plain(ks)) cs = row_scales(ks);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        double2 u = value(ks, 0, i);
+        const unsigned c = unsigned(i < 2 ? (i == 0 ? cs.x : cs.y) : (i == 2 ? cs.z : cs.w));
+        const double2 u = value(ks, 0, i);
         if constexpr (FOLD) {
-          if (i == 0 && a.wall && ks == 0 && t == 0) u = make_double2(0.0, 0.0);
           const double2 v = value(ks, 1, i);
-          const Fixed u0 = to_fixed(u.x, emax0), v0 = to_fixed(v.x, emax0);
-          const Fixed u1 = to_fixed(u.y, emax1), v1 = to_fixed(v.y, emax1);
+          const Fixed u0 = to_fixed(u.x, top0 + c), v0 = to_fixed(v.x, top0 + c);
+          const Fixed u1 = to_fixed(u.y, top1 + c), v1 = to_fixed(v.y, top1 + c);
           P[i][0] = fixed_sum(u0, v0); Q[i][0] = fixed_difference(u0, v0);
           P[i][1] = fixed_sum(u1, v1); Q[i][1] = fixed_difference(u1, v1);
         } else {
-          P[i][0] = fixed_value(to_fixed(u.x, emax0));
-          P[i][1] = fixed_value(to_fixed(u.y, emax1));
+          P[i][0] = fixed_value(to_fixed(u.x, top0 + c));
+          P[i][1] = fixed_value(to_fixed(u.y, top1 + c));
         }
       }
       __syncwarp();                                    // every lane has this step's values
@@ -427,7 +473,8 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 3) split_contract_kernel(con
 #pragma unroll 1
     for (int ks = n0 + s1 - s0; ks < n1; ++ks) copy(unit2, ks);     // a longer run follows
     // V 2^-8 = acc_0 2^37 + acc_1 2^28 + acc_2 2^19 + (acc_3 2^18 + acc_4 2^9 + acc_5) 2^-8
-    const Exponent e0(emax0 - 1075 - (tiny0 ? 128 : 0)), e1(emax1 - 1075 - (tiny1 ? 128 : 0));
+    const Exponent e0(emax0 - 1075 - (tiny0 ? 128 : 0), emax0 < 0x7ff), e1(emax1 - 1075 - (tiny1 ? 128 : 0), emax1 < 0x7ff);
+    const bool rare = __any_sync(0xffffffffu, (e0.extra | e1.extra) != 0);    // (the same for the warp: no divergence)
     const int o = unit / a.ztiles;
     double* out = a.out + size_t(o) * a.out_o + (unit - o * a.ztiles) * 16 + 2 * g;
 #pragma unroll
@@ -446,9 +493,8 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 3) split_contract_kernel(con
         if (q < (FOLD ? half : a.rows)) {
           double2* p = reinterpret_cast<double2*>(out + size_t(r) * a.out_r);
           double2 w = make_double2(0.0, 0.0);
-          if (!zero) w = make_double2(to_double<false>(fixed(c), e0.e), to_double<true>(fixed(2 + c), e1.e));
-          if (e0.extra | e1.extra) w = rescale(w, e0.extra, e1.extra);
-          w = nan_where(w, emax0, emax1);
+          if (!zero) w = make_double2(to_double<false>(fixed(c), e0.e20), to_double<true>(fixed(2 + c), e1.e20));
+          if (rare) w = rescale(w, e0.extra, e1.extra);
           if (s0 > 0) {
             const double2 b = *p;
             w.x += b.x;
@@ -473,6 +519,7 @@ struct ExpandArgs {
   const double* in;          // value (o, k, z) at o * in_o + k * in_k + z
   double* out;               // value (o, r, z) at o * out_o + r * out_r + z
   const uint4* tab;
+  RowScale scale;            // of the output rows
   size_t in_o, in_k, out_o, out_r;
   int outer, ztiles;
   int K;                     // modes (FOLD: both halves)
@@ -499,7 +546,7 @@ __device__ __forceinline__ void digits_round(unsigned long long a, unsigned long
 }
 
 template <int KS, bool FOLD, bool SMALL>
-__global__ void __launch_bounds__(32 * kSplitWarps, 3) split_expand_kernel(const __grid_constant__ ExpandArgs a) {
+__global__ void __launch_bounds__(32 * kSplitWarps, FOLD ? 4 : (KS == 2 ? 5 : 7)) split_expand_kernel(const __grid_constant__ ExpandArgs a) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int unit = int(blockIdx.x) * kSplitWarps + (int(threadIdx.x) >> 5);
   if (unit >= a.outer * a.ztiles) return;
@@ -535,7 +582,7 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 3) split_expand_kernel(const
       for (int i = 0; i < 4; ++i) x[ks][i] = raise(x[ks][i], tiny0, tiny1);
     top = largest();
   }
-  const int emax0 = max(int(top.x >> 20), kTiny), emax1 = max(int(top.y >> 20), kTiny);
+  const int emax0 = exponent_of(top.x), emax1 = exponent_of(top.y);
   unsigned A[KS][kD][4];
 #pragma unroll
   for (int ks = 0; ks < KS; ++ks)
@@ -550,7 +597,9 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 3) split_expand_kernel(const
 #pragma unroll
       for (int i = 0; i < kD; ++i) A[ks][i][2 * h + 1] = d[i];
     }
-  const Exponent e0(emax0 - 1083 - kExtra + 6 - (tiny0 ? 128 : 0)), e1(emax1 - 1083 - kExtra + 6 - (tiny1 ? 128 : 0));
+  const Exponent e0(emax0 - 1083 - kExtra + 6 - (tiny0 ? 128 : 0), emax0 < 0x7ff);
+  const Exponent e1(emax1 - 1083 - kExtra + 6 - (tiny1 ? 128 : 0), emax1 < 0x7ff);
+  const bool rare = __any_sync(0xffffffffu, (e0.extra | e1.extra) != 0);      // (the same for the warp: no divergence)
   // V 2^-6 = acc_0 2^39 + acc_1 2^30 + acc_2 2^21 + acc_3 2^12 + acc_4 2^3 + acc_5 2^-6,
   // without kOff where the sums are read off with their offset M
   constexpr unsigned M = 0x4B400000u;                // the bits of 1.5 2^23
@@ -583,50 +632,51 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 3) split_expand_kernel(const
       if (ks % KH == 0) mma_split<true>(acc[ks / KH], A[ks], tb + ks * (kD / 2) * 32, SMALL ? 12582912.f : 0.f);
       else mma_split<false>(acc[ks / KH], A[ks], tb + ks * (kD / 2) * 32);
     }
+    const int2 scale = __ldg(reinterpret_cast<const int2*>(a.scale.rows + 16 * (tile >> 1) + 4 * t + 2 * (tile & 1)));
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       const int r = 8 * tile + 2 * t + c;
+      const int x0 = e0.e20 - (c ? scale.y : scale.x), x1 = e1.e20 - (c ? scale.y : scale.x);
       const unsigned long long o0 = fixed(acc[0], c), o1 = fixed(acc[0], 2 + c);
       if constexpr (FOLD) {
         const unsigned long long v0 = fixed(acc[1], c), v1 = fixed(acc[1], 2 + c);
-        double2 lo = make_double2(to_double<false>(static_cast<long long>(o0 + v0 - 2 * kOff), e0.e),
-                                  to_double<false>(static_cast<long long>(o1 + v1 - 2 * kOff), e1.e));
-        double2 hi = make_double2(to_double<true>(static_cast<long long>(o0 - v0), e0.e),
-                                  to_double<true>(static_cast<long long>(o1 - v1), e1.e));
-        if (e0.extra | e1.extra) {
+        double2 lo = make_double2(to_double<false>(static_cast<long long>(o0 + v0 - 2 * kOff), x0),
+                                  to_double<false>(static_cast<long long>(o1 + v1 - 2 * kOff), x1));
+        double2 hi = make_double2(to_double<true>(static_cast<long long>(o0 - v0), x0),
+                                  to_double<true>(static_cast<long long>(o1 - v1), x1));
+        const bool on_wall = a.wall && r == 0;
+        if (on_wall) lo = make_double2(0.0, 0.0);
+        if (rare) {
           lo = rescale(lo, e0.extra, e1.extra);
           hi = rescale(hi, e0.extra, e1.extra);
         }
-        const bool on_wall = a.wall && r == 0;
-        if (on_wall) lo = make_double2(0.0, 0.0);
-        lo = nan_where(lo, emax0, emax1);
-        hi = nan_where(hi, emax0, emax1);
         *reinterpret_cast<double2*>(out + size_t(r) * a.out_r) = lo;
         *reinterpret_cast<double2*>(out + size_t(on_wall ? a.wall : a.mirror - r) * a.out_r) = hi;
       } else {
-        double2 v = make_double2(to_double<false>(static_cast<long long>(o0 - kOff), e0.e),
-                                 to_double<true>(static_cast<long long>(o1 - kOff), e1.e));
-        if (e0.extra | e1.extra) v = rescale(v, e0.extra, e1.extra);
-        *reinterpret_cast<double2*>(out + size_t(r) * a.out_r) = nan_where(v, emax0, emax1);
+        double2 v = make_double2(to_double<false>(static_cast<long long>(o0 - kOff), x0),
+                                 to_double<true>(static_cast<long long>(o1 - kOff), x1));
+        if (rare) v = rescale(v, e0.extra, e1.extra);
+        *reinterpret_cast<double2*>(out + size_t(r) * a.out_r) = v;
       }
     }
   }
 }
 
 // Fragments of a table tab[rows][slots] (|values| <= 1), digits of
-// round(value 2^53).  contract: [k step over rows][tile of 8 slots][digit
+// round(value 2^(53 + the row's scale)).  contract: [k step over rows][tile of 8 slots][digit
 // pair][lane]; expand: [tile of 8 rows][k step over slots][digit pair][lane].
 // A piece is (b0, b1) of digit 2i, then of digit 2i + 1; b0 holds k = 2t,
 // 2t + 1 and b1 k = 2t + 8, 2t + 9 of column g.
-__device__ __forceinline__ unsigned short table_digit(const double* tab, int rows, int slots, int row, int slot,
-                                                      int digit) {
+__device__ __forceinline__ unsigned short table_digit(const double* tab, const int* scale, int rows, int slots, int row,
+                                                      int slot, int digit) {
   if (row >= rows || slot < 0 || slot >= slots) return 0;
-  const long long X = __double2ll_rn(tab[size_t(row) * slots + slot] * 0x1p53) + kBias;
+  const int s = min(scale[scale_index(row)] >> 20, kMaxRowScale);        // (kZeroRow: only zeros there)
+  const long long X = __double2ll_rn(ldexp(tab[size_t(row) * slots + slot], 53 + s)) + kBias;
   const int f = digit == 0 ? int(X >> 45) - 512 : int((X >> (kB * (kD - 1 - digit))) & 511) - 256;
   return __half_as_ushort(__int2half_rn(f));
 }
 
-__global__ void split_table_kernel(const double* tab, int rows, int slots, int halves, int expand, uint4* out,
+__global__ void split_table_kernel(const double* tab, const int* scale, int rows, int slots, int halves, int expand, uint4* out,
                                    long total) {
   const long idx = long(blockIdx.x) * blockDim.x + threadIdx.x;
   if (idx >= total) return;
@@ -656,7 +706,7 @@ __global__ void split_table_kernel(const double* tab, int rows, int slots, int h
       const int row = expand ? n : k;
       int slot = base + (expand ? k : n);
       if (slot >= limit) slot = -1;
-      h[c] = table_digit(tab, rows, slots, row, slot, 2 * dp + (w >> 1));
+      h[c] = table_digit(tab, scale, rows, slots, row, slot, 2 * dp + (w >> 1));
     }
     r[w] = unsigned(h[0]) | unsigned(h[1]) << 16;
   }
@@ -706,23 +756,46 @@ cudaError_t expand(const ExpandArgs& a, bool fold, bool small, cudaStream_t st) 
 
 }  // namespace
 
-cudaError_t build_split_table(const double* tab, int rows, int slots, bool halves, bool expand, uint4* out,
-                              cudaStream_t st) {
+cudaError_t build_split_table(const double* tab, const int* scale, int rows, int slots, bool halves, bool expand,
+                              uint4* out, cudaStream_t st) {
   const long total = long(expand ? split_expand_size(rows, slots, halves) : split_contract_size(rows, slots, halves));
-  split_table_kernel<<<unsigned((total + 127) / 128), 128, 0, st>>>(tab, rows, slots, halves, expand, out, total);
+  split_table_kernel<<<unsigned((total + 127) / 128), 128, 0, st>>>(tab, scale, rows, slots, halves, expand, out, total);
   return cudaGetLastError();
+}
+
+// the power of two that brings a row's largest value into [1/2, 1]
+RowScale table_scales(const double* tab, int rows, int slots, int* scale) {
+  for (int r = 0; r < split_padded(rows); ++r) {
+    double top = 0.0;
+    for (int k = 0; r < rows && k < slots; ++k) top = std::fmax(top, std::fabs(tab[size_t(r) * slots + k]));
+    int e = 0;
+    if (top > 0.0) std::frexp(top, &e);
+    const int s = top > 0.0 ? std::min(std::max(-e, 0), kMaxRowScale) : kZeroRow;
+    scale[scale_index(r)] = s * (1 << 20);
+  }
+  RowScale out{nullptr, 0, 0};                       // the longest run of steps without a scale
+  for (int k = 0, from = 0; k < split_padded(rows) / 16; ++k) {
+    for (int r = 16 * k; r < 16 * k + 16 && r < rows; ++r)
+      if (scale[scale_index(r)] != 0) from = k + 1;
+    if (k + 1 - from > out.plain1 - out.plain0) {
+      out.plain0 = from;
+      out.plain1 = k + 1;
+    }
+  }
+  return out;
 }
 
 // sum over j of (the largest |d_{s-j}|) sum_k |t_j| below 2^22 for every table
 // row, half and weight s: the expansion's sums can be read off the bits
-bool expand_sums_small(const double* tab, int rows, int slots, bool halves) {
+bool expand_sums_small(const double* tab, const int* scale, int rows, int slots, bool halves) {
   const int kh = halves ? slots / 2 : slots;
   if (kh > 16) return false;
   for (int r = 0; r < rows; ++r)
     for (int h = 0; h < (halves ? 2 : 1); ++h) {
       long sum[kD] = {};
       for (int k = 0; k < kh; ++k) {
-        const long long X = std::llrint(tab[size_t(r) * slots + h * kh + k] * 0x1p53) + kBias;
+        const int s = std::min(scale[scale_index(r)] >> 20, kMaxRowScale);
+        const long long X = std::llrint(std::ldexp(tab[size_t(r) * slots + h * kh + k], 53 + s)) + kBias;
         for (int j = 0; j < kD; ++j) {
           const long f = j == 0 ? long(X >> 45) - 512 : long((X >> (kB * (kD - 1 - j))) & 511) - 256;
           sum[j] += f < 0 ? -f : f;
@@ -748,6 +821,7 @@ cudaError_t launch_split_project(const SplitArgs& s, const double* rho, double* 
     y.out_o = size_t(s.myp) * s.zs;
     y.out_r = size_t(s.zs);
     y.tab = s.cy;
+    y.scale = s.ys;
     y.outer = s.nx;
     y.ztiles = s.zs / 16;
     y.K = fold ? s.ny / 2 : s.ny;
@@ -765,6 +839,7 @@ cudaError_t launch_split_project(const SplitArgs& s, const double* rho, double* 
     x.out_o = size_t(s.nz);
     x.out_r = size_t(s.myp) * s.nz;
     x.tab = s.cx;
+    x.scale = s.xs;
     x.outer = s.myp;
     x.ztiles = s.zs / 16;
     x.K = s.nx;
@@ -786,6 +861,7 @@ cudaError_t launch_split_back(const SplitArgs& s, const double* psi, double* phi
     x.out_o = size_t(s.zs);
     x.out_r = size_t(s.myp) * s.zs;
     x.tab = s.ex;
+    x.scale = s.xs;
     x.outer = s.myp;
     x.ztiles = s.zs / 16;
     x.K = s.mxp;
@@ -801,6 +877,7 @@ cudaError_t launch_split_back(const SplitArgs& s, const double* psi, double* phi
     y.out_o = size_t(s.ny) * s.nz;
     y.out_r = size_t(s.nz);
     y.tab = s.ey;
+    y.scale = s.ys;
     y.outer = s.nx;
     y.ztiles = s.zs / 16;
     y.K = s.myp;

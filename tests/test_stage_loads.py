@@ -12,7 +12,7 @@ TABLES = {
     "modes.cu": set(),
     "modes_z.cu": {"zp"},                       # z recurrences
     "modes_sums.cu": {"sy", "p", "a.sx"},       # sine tables (p: a row of the y table)
-    "modes_split.cu": {"tb"},                   # digit fragments
+    "modes_split.cu": {"tb", "a.scale.rows"},        # digit fragments, row scales
     "zfft_impl.cuh": {"w2", "a.w2_z"},          # phases
     "tdst_impl.cuh": {"tw", "grow"},            # twiddles, Green spectrum
     "fft_common.cuh": {"tw"},
