@@ -303,6 +303,7 @@ int mode_stage(const pipe_handle* h, int stage, const void* rho, void* phi, void
     SplitArgs s{};
     s.cy = h->mcy; s.cx = h->mcx; s.ey = h->mey; s.ex = h->mex;
     s.ys = h->mys; s.xs = h->mxs;
+    s.cy_run = h->mcy_run; s.cx_run = h->mcx_run;
     s.ey_small = h->mey_small; s.ex_small = h->mex_small;
     s.nx = a.nx; s.ny = a.ny; s.nz = a.nz;
     s.mx = a.mx; s.mxp = h->mxp; s.myp = h->myp;
@@ -503,11 +504,13 @@ static int setup_pipe(const pipe_geometry* geom, const pipe_grid* grid, int igf,
       e = cudaMemcpy(t, h->msy64, nsy * sizeof(double), cudaMemcpyDeviceToHost);
       if (e == cudaSuccess) {
         h->mys = table_scales(t, nyk, h->myp, scale);
+        h->mcy_run = contract_steps(t, scale, nyk, h->myp, halves);
         h->mey_small = expand_sums_small(t, scale, nyk, h->myp, halves);
         e = cudaMemcpy(t, h->msx64, nsx * sizeof(double), cudaMemcpyDeviceToHost);
       }
       if (e == cudaSuccess) {
         h->mxs = table_scales(t, grid->nx, h->mxp, scale + npy);
+        h->mcx_run = contract_steps(t, scale + npy, grid->nx, h->mxp, false);
         h->mex_small = expand_sums_small(t, scale + npy, grid->nx, h->mxp, false);
         e = cudaMemcpy(rows, scale, size_t(npy + npx) * sizeof(int), cudaMemcpyHostToDevice);
       }

@@ -69,6 +69,7 @@ struct pipe_handle {
   uint4* msplit = nullptr;
   uint4 *mcy = nullptr, *mcx = nullptr, *mey = nullptr, *mex = nullptr;
   pp::RowScale mys{}, mxs{};                   // the tables' row scales (in the same allocation)
+  int mcy_run = 1, mcx_run = 1;                // contract_steps of mcy, mcx
   bool mey_small = false, mex_small = false;   // expand_sums_small of mey, mex
   // part [groups][mc][nz], then psi [mc][nz], of the dtype; FP64: then the
   // half-transformed field of a slab (modes_split.cuh)

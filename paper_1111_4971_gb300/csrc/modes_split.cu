@@ -8,14 +8,15 @@
 // Rump, "Error-free transformations of matrix multiplication by using fast
 // routines of matrix multiplication", 2012), each digit a small integer that
 // FP16 holds exactly.  Digit products are summed by FP16 MMA with FP32
-// accumulators, exactly: a digit product is at most 2^16 (2^17 for the leading
-// digit of a folded pair), a sum over at most 64 rows and the 1 to 6 products
-// of one weight stays below 2^24 (for the two smallest weights, whose last bit
-// is below 2^-57 of the result, only barring an adversarial choice of every
-// digit at once).  The products d_i t_j with i + j <= 5 are kept, 21 of 36:
-// what is dropped is below 2^-54 of the largest term, the rounding of one FP64
-// product.  The six sums are put together in 64-bit integers and rounded to
-// FP64 once.  No FP64 arithmetic is left but one addition per 64 rows.
+// accumulators.  The products d_i t_j with i + j <= 5 are kept, 21 of 36: each one
+// dropped is below 2^-54 of the largest term, the rounding of one FP64 product.
+// The sums of the weights i + j = 0 .. 4 are exact, at most 2^24: how many rows go
+// into one set of accumulators, 64 unless a table's digits are all large, follows
+// from the table (contract_steps; |d_i| <= 256, |d_0| <= 512 for a folded pair); the
+// expansion has 16 terms (32 unfolded, 32 (1024 + 4 256) 256 <= 2^24).  Those of weight
+// 5 may pass 2^24 and lose their last bit, 2^-61 of a largest term.  The six sums
+// are put together in 64-bit integers and rounded to FP64 once; half of the
+// outputs are converted on the FP64 pipe, which else adds once per 64 rows.
 //
 // Two kernels, used for y and for x in turn; one warp per (outer index, 16
 // consecutive z), no barrier beyond the warp:
@@ -58,8 +59,6 @@
 // run by itself, pipe_stage_modes: of their 16 planes).
 #include <cuda_fp16.h>
 
-#include <algorithm>
-#include <cmath>
 #include <utility>
 
 #include "modes_impl.cuh"
@@ -69,14 +68,11 @@ namespace pp {
 
 namespace {
 
-constexpr int kD = kSplitDigits, kB = kSplitBits;
+constexpr int kD = kSplitDigits;
 constexpr int kSplitWarps = 4;                       // warps per CTA
-constexpr int kSeg = 64;                             // rows summed in one set of accumulators
+constexpr int kSeg = 64;                             // rows of a warp's tile
 
-// Biased values: X + bias has the non-negative 9-bit fields d_i + 256 (i = 5 .. 1)
-// and d_0 + (a multiple of 512) above them
-constexpr long long kBiasLow = 256LL * (1 + (1LL << 9) + (1LL << 18) + (1LL << 27) + (1LL << 36));
-constexpr long long kBias = kBiasLow + (512LL << 45);
+constexpr long long kBiasLow = kSplitBiasLow, kBias = kSplitBias;
 // a contraction's values keep kGuard more bits until their digits are taken, and
 // are rounded there: cut off, they would all move towards zero, an error that a
 // sum does not average out
@@ -281,6 +277,7 @@ struct ContractArgs {
   size_t in_o, in_k, out_o, out_r;
   int outer, ztiles;         // units: outer x ztiles, 16 z each
   int K;                     // rows, or mirror pairs
+  int run;                   // 16-row steps summed in one set of accumulators (contract_steps)
   int rows;                  // output rows (slots)
   int mirror;                // FOLD: row k's mirror is row mirror - k
   int wall;                  // FOLD: pair 0 is row 0 (on the wall, table zero) and row `wall`
@@ -312,8 +309,9 @@ __device__ __forceinline__ void copy_step(const ContractArgs& a, int unit, int k
   cp_async_commit();
 }
 
-// Persistent: a warp takes the runs (unit, at most kSeg rows) of the units
-// w, w + warps, ..; as soon as a k step's values are in registers, the same
+// Persistent: a warp takes the runs (unit, at most a.run steps) of the units
+// w, w + warps, ..; a.run divides the tile's 4 steps, so that a step's place in the
+// tile is never one that the run in progress has still to read; as soon as a k step's values are in registers, the same
 // step of its next run is copied over them (cp.async), so that a run's loads
 // from memory overlap the digits and products of the one before.
 template <int NT, bool FOLD>
@@ -344,13 +342,13 @@ __global__ void __launch_bounds__(32 * kSplitWarps, 3) split_contract_kernel(con
   int unit = int(blockIdx.x) * kSplitWarps + warp, s0 = 0;
   wait_stage();
   if (unit < units)
-    for (int ks = 0; ks < min(kSeg / 16, steps); ++ks) copy(unit, ks);
+    for (int ks = 0; ks < min(a.run, steps); ++ks) copy(unit, ks);
 #pragma unroll 1
   while (unit < units) {
-    const int s1 = min(s0 + kSeg / 16, steps);
+    const int s1 = min(s0 + a.run, steps);
     // the run after this one
     const int unit2 = s1 < steps ? unit : unit + stride, n0 = s1 < steps ? s1 : 0;
-    const int n1 = unit2 < units ? min(n0 + kSeg / 16, steps) : n0;
+    const int n1 = unit2 < units ? min(n0 + a.run, steps) : n0;
     cp_async_wait<0>();
     __syncwarp();
     // per plane, the largest high word of the values, each less its row's scale (a
@@ -671,9 +669,8 @@ __device__ __forceinline__ unsigned short table_digit(const double* tab, const i
                                                       int slot, int digit) {
   if (row >= rows || slot < 0 || slot >= slots) return 0;
   const int s = min(scale[scale_index(row)] >> 20, kMaxRowScale);        // (kZeroRow: only zeros there)
-  const long long X = __double2ll_rn(ldexp(tab[size_t(row) * slots + slot], 53 + s)) + kBias;
-  const int f = digit == 0 ? int(X >> 45) - 512 : int((X >> (kB * (kD - 1 - digit))) & 511) - 256;
-  return __half_as_ushort(__int2half_rn(f));
+  const long long X = __double2ll_rn(ldexp(tab[size_t(row) * slots + slot], 53 + s));
+  return __half_as_ushort(__int2half_rn(split_digit(X, digit)));
 }
 
 __global__ void split_table_kernel(const double* tab, const int* scale, int rows, int slots, int halves, int expand, uint4* out,
@@ -763,53 +760,6 @@ cudaError_t build_split_table(const double* tab, const int* scale, int rows, int
   return cudaGetLastError();
 }
 
-// the power of two that brings a row's largest value into [1/2, 1]
-RowScale table_scales(const double* tab, int rows, int slots, int* scale) {
-  for (int r = 0; r < split_padded(rows); ++r) {
-    double top = 0.0;
-    for (int k = 0; r < rows && k < slots; ++k) top = std::fmax(top, std::fabs(tab[size_t(r) * slots + k]));
-    int e = 0;
-    if (top > 0.0) std::frexp(top, &e);
-    const int s = top > 0.0 ? std::min(std::max(-e, 0), kMaxRowScale) : kZeroRow;
-    scale[scale_index(r)] = s * (1 << 20);
-  }
-  RowScale out{nullptr, 0, 0};                       // the longest run of steps without a scale
-  for (int k = 0, from = 0; k < split_padded(rows) / 16; ++k) {
-    for (int r = 16 * k; r < 16 * k + 16 && r < rows; ++r)
-      if (scale[scale_index(r)] != 0) from = k + 1;
-    if (k + 1 - from > out.plain1 - out.plain0) {
-      out.plain0 = from;
-      out.plain1 = k + 1;
-    }
-  }
-  return out;
-}
-
-// sum over j of (the largest |d_{s-j}|) sum_k |t_j| below 2^22 for every table
-// row, half and weight s: the expansion's sums can be read off the bits
-bool expand_sums_small(const double* tab, const int* scale, int rows, int slots, bool halves) {
-  const int kh = halves ? slots / 2 : slots;
-  if (kh > 16) return false;
-  for (int r = 0; r < rows; ++r)
-    for (int h = 0; h < (halves ? 2 : 1); ++h) {
-      long sum[kD] = {};
-      for (int k = 0; k < kh; ++k) {
-        const int s = std::min(scale[scale_index(r)] >> 20, kMaxRowScale);
-        const long long X = std::llrint(std::ldexp(tab[size_t(r) * slots + h * kh + k], 53 + s)) + kBias;
-        for (int j = 0; j < kD; ++j) {
-          const long f = j == 0 ? long(X >> 45) - 512 : long((X >> (kB * (kD - 1 - j))) & 511) - 256;
-          sum[j] += f < 0 ? -f : f;
-        }
-      }
-      for (int w = 0; w < kD; ++w) {
-        long bound = 0;
-        for (int j = 0; j <= w; ++j) bound += sum[j] * (w - j == 0 ? 256L << kExtra : 256L);
-        if (bound >= 1L << 22) return false;
-      }
-    }
-  return true;
-}
-
 cudaError_t launch_split_project(const SplitArgs& s, const double* rho, double* part, cudaStream_t st) {
   const bool fold = s.fold != 0;
   for (int z0 = 0; z0 < s.nz; z0 += s.zs) {
@@ -821,6 +771,7 @@ cudaError_t launch_split_project(const SplitArgs& s, const double* rho, double* 
     y.out_o = size_t(s.myp) * s.zs;
     y.out_r = size_t(s.zs);
     y.tab = s.cy;
+    y.run = s.cy_run;
     y.scale = s.ys;
     y.outer = s.nx;
     y.ztiles = s.zs / 16;
@@ -839,6 +790,7 @@ cudaError_t launch_split_project(const SplitArgs& s, const double* rho, double* 
     x.out_o = size_t(s.nz);
     x.out_r = size_t(s.myp) * s.nz;
     x.tab = s.cx;
+    x.run = s.cx_run;
     x.scale = s.xs;
     x.outer = s.myp;
     x.ztiles = s.zs / 16;

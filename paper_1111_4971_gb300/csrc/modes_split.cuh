@@ -6,11 +6,9 @@
 #include <cstddef>
 #include <cstdint>
 
-namespace pp {
+#include "split_tables.h"
 
-// Digits of a split value, and products kept per pair of split values.
-constexpr int kSplitDigits = 6;
-constexpr int kSplitBits = 9;
+namespace pp {
 
 // Fragment tables of one sine table (see split_table_kernel): uint4 values
 inline int split_tiles(int n) { return (n + 7) / 8; }       // columns of 8
@@ -28,25 +26,9 @@ inline int split_expand_steps(int slots, bool halves) { return halves ? 2 * spli
 inline size_t split_expand_size(int rows, int slots, bool halves) {
   return size_t(split_tiles(rows)) * split_expand_steps(slots, halves) * (kSplitDigits / 2) * 32;
 }
-// A table row's scale: its digits are those of the row times 2^s, 0 <= s <=
-// kMaxRowScale, or kZeroRow where the row is zero; stored as s 2^20 (an FP64
-// number's exponent is there in its high word), for rows padded to a multiple of 16
-constexpr int kMaxRowScale = 64, kZeroRow = 2047;
-// row r's place: 16 rows are kept as a lane's four, 2t, 2t + 1, 2t + 8, 2t + 9, for t = 0 .. 3
-__host__ __device__ inline int scale_index(int r) { return r / 16 * 16 + (r % 8) / 2 * 4 + (r % 16) / 8 * 2 + r % 2; }
-inline int split_padded(int rows) { return (rows + 15) / 16 * 16; }
-struct RowScale {
-  const int* rows;
-  int plain0, plain1;        // 16-row steps of the table in which every scale is 0
-};
-RowScale table_scales(const double* tab, int rows, int slots, int* scale);     // host memory; .rows is left null
-
 // tab [rows][slots] and scale in device memory
 cudaError_t build_split_table(const double* tab, const int* scale, int rows, int slots, bool halves, bool expand,
                               uint4* out, cudaStream_t st);
-
-// the expansion over this table [rows][slots] (host memory) can take its sums off the accumulators' bits
-bool expand_sums_small(const double* tab, const int* scale, int rows, int slots, bool halves);
 
 // One FP64 solve's stages: tables, mesh and the buffer of the half-transformed
 // field [nx][myp][zs] (zs z values at a time, split_slab)
@@ -54,7 +36,8 @@ struct SplitArgs {
   const uint4 *cy, *cx;      // contraction tables of the y modes and the x modes
   const uint4 *ey, *ex;      // expansion tables
   RowScale ys, xs;           // the tables' row scales
-  bool ey_small, ex_small;   // expand_sums_small of them
+  int cy_run, cx_run;        // contract_steps of cy, cx
+  bool ey_small, ex_small;   // expand_sums_small of ey, ex
   int nx, ny, nz;
   int mx, mxp, myp;
   int fold;                  // 0: all rows, 1: mirror pairs (j, ny-1-j), 2: (j, ny-j) with row 0 on the wall

@@ -6,7 +6,7 @@ import torch
 
 from inputs.bunches import Geometry, Grid
 from test_gpu_mode_split import make
-from test_gpu_mode_split_planes import back, project, tables
+from test_gpu_mode_split_planes import back, project, sinpi, tables
 
 pytestmark = pytest.mark.gpu
 
@@ -78,3 +78,34 @@ def test_density_on_the_wall_is_not_felt(dtype):
         r[0] = scale
         r[:, 0] = -scale
         assert torch.equal(s.solve(r), want)
+
+
+def test_tables_that_sum_fewer_rows_at_a_time():
+    """A window so narrow that a mode's sines agree in every row and all their
+    digits are large: 64 such rows pass what the accumulators hold exactly, so the
+    contraction over y takes 32 at a time."""
+    from paper_1111_4971_gb300 import PipeSolver
+    n = np.arange(1, 33)
+
+    def digits(t):
+        x = int(np.rint(np.ldexp(t, 53 + max(0, -int(np.frexp(abs(t))[1])))))
+        out = []
+        for _ in range(5):
+            out.append((x + 256) % 512 - 256)
+            x = (x - out[-1]) // 512
+        return np.abs([x] + out[::-1])
+
+    def heaviest(y0):
+        return max(digits(float(t))[:5].sum() for t in sinpi(n.astype(np.float64) * y0))
+
+    y0 = max((k / 997 for k in range(100, 400)), key=heaviest)
+    assert 64 * 256 * heaviest(y0) > 1.02 * 2 ** 24
+    nx, ny, nz = 16, 80, 32
+    s = PipeSolver(Geometry(1.3, 1.0, 0.05, y0, 6, 32), Grid(nx, ny, nz, 0.07, 1e-19, 0.05), igf=True, dtype=torch.float64)
+    s.set_plan(t_kind=3)
+    sx, sy = tables(s)
+    g = torch.Generator(device="cuda").manual_seed(2)
+    rho = torch.rand(nx, ny, nz, dtype=torch.float64, device="cuda", generator=g) - 0.3
+    part, psi = s.mode_buffers()
+    s.stage_modes(0, rho, part)
+    assert ((part.sum(0) - project(sx, sy, rho)).abs() <= 16 * U * nx * ny).all()
