@@ -367,10 +367,12 @@ int pipe_mode_spectrum(pipe_handle* h, double* out, size_t count);
  * t_kind 3); it is symmetric, so the adjoint is the same chain.
  * FP64: a value of stage 0's or stage 2's input that is not finite makes the
  * outputs of its tile of 16 z planes NaN (in a solve: of its own z plane).
- * FP64 stages 0 and 2 keep the half-transformed field in the handle's
- * workspace, as a solve does: one such call or solve per handle at a time.
+ * A stage touches the caller's buffers only, so it may run beside a solve or
+ * another stage of the handle on another stream.  FP64 stages 0 and 2 take
+ * nx*myp*nz values (at most 32 MiB) from the device's memory pool for the call,
+ * in stream order.
  * Errors: PIPE_EINVAL (stage outside 0..2, null or misaligned pointers),
- * PIPE_EUNSUPPORTED as pipe_mode_layout, PIPE_ECUDA. */
+ * PIPE_EUNSUPPORTED as pipe_mode_layout, PIPE_ENOMEM, PIPE_ECUDA. */
 int pipe_stage_modes(pipe_handle* h, int stage, const void* in, void* out, void* stream);
 
 /* Time the kernel variants available for this handle's sizes on `stream` and

@@ -779,9 +779,17 @@ int pipe_stage_modes(pipe_handle* h, int stage, const void* in, void* out, void*
   void* psi = stage == 1 ? out : (stage == 2 ? vin : nullptr);
   void* phi = stage == 2 ? out : nullptr;
   if (h->grid.dtype != PIPE_F64) return mode_stage<float>(h, stage, rho, phi, part, psi, nullptr, true, s);
-  // the half-transformed field is the handle's, as in a solve
-  char* half = static_cast<char*>(h->mwork) + sizeof(double) * size_t(mode_xblocks(h) + 1) * h->mxp * h->myp * h->grid.nz;
-  return mode_stage<double>(h, stage, rho, phi, part, psi, half, true, s);
+  if (stage == 1) return mode_stage<double>(h, stage, rho, phi, part, psi, nullptr, true, s);
+  // the half-transformed field: a buffer of this call alone, in stream order, so
+  // that a stage may run beside a solve or another stage of the same handle
+  void* half = nullptr;
+  const cudaError_t e = cudaMallocAsync(&half, split_half_bytes(h->grid.nx, h->myp, h->grid.nz), s);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return e == cudaErrorMemoryAllocation ? PIPE_ENOMEM : PIPE_ECUDA;
+  }
+  st = mode_stage<double>(h, stage, rho, phi, part, psi, half, true, s);
+  return cudaFreeAsync(half, s) == cudaSuccess ? st : PIPE_ECUDA;
 }
 
 }  // extern "C"
