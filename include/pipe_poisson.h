@@ -347,7 +347,9 @@ int pipe_mode_layout(pipe_handle* h, int* mx, int* mxp, int* myp, int* fold, int
  * (f = exp(-kappa |w|) of Eq. 9, or the IGF g_z of Eq. 15), with the free
  * slot d = nz filled by the formula, divided by 2*nz; zero for padded
  * columns.  count must be mxp*myp*(nz+1).  Synchronous.  For inspection and
- * tests.  Errors: PIPE_EINVAL, PIPE_EUNSUPPORTED as pipe_mode_layout. */
+ * tests: the table is computed at a handle's first call and kept until it is
+ * destroyed, later calls are a copy.  Errors: PIPE_EINVAL, PIPE_ENOMEM,
+ * PIPE_EUNSUPPORTED as pipe_mode_layout. */
 int pipe_mode_spectrum(pipe_handle* h, double* out, size_t count);
 
 /* Stages of the mode-space form, for inspection and per-kernel tests (device

@@ -127,6 +127,7 @@ void free_handle(pipe_handle* h) {
   cudaFree(h->msx64); cudaFree(h->msy64);
   cudaFree(h->msx32); cudaFree(h->msy32);
   cudaFree(h->mzp64); cudaFree(h->mzp32);
+  cudaFree(h->mgz64);
   cudaFree(h->mwork);
   cudaFree(h->msplit);
   cudaFree(h->mkb64); cudaFree(h->mkb32);
@@ -749,17 +750,24 @@ int pipe_mode_spectrum(pipe_handle* h, double* out, size_t count) {
   if (!h->modes_ok) return PIPE_EUNSUPPORTED;
   if (count != size_t(h->mxp) * h->myp * (h->grid.nz + 1)) return PIPE_EINVAL;
   DeviceGuard dg(h->device);
-  GreenSpec s{};
-  s.nx = h->grid.nx; s.ny = h->grid.ny; s.nz = h->grid.nz;
-  s.hx = h->grid.hx; s.hy = h->grid.hy; s.hz = h->grid.hz;
-  s.a = h->geom.a; s.b = h->geom.b;
-  s.modes_m = h->geom.modes_m; s.modes_n = h->geom.modes_n;
-  s.igf = h->kind;
-  double* g = nullptr;
-  cudaError_t e = cudaMalloc(&g, count * sizeof(double));
-  if (e == cudaSuccess) e = build_mode_spectrum(s, h->mxp, h->myp, h->fy, g, nullptr);
-  if (e == cudaSuccess) e = cudaMemcpy(out, g, count * sizeof(double), cudaMemcpyDeviceToHost);
-  cudaFree(g);
+  cudaError_t e = cudaSuccess;
+  {
+    std::lock_guard<std::mutex> lk(h->mgz_mu);
+    if (!h->mgz64) {
+      GreenSpec s{};
+      s.nx = h->grid.nx; s.ny = h->grid.ny; s.nz = h->grid.nz;
+      s.hx = h->grid.hx; s.hy = h->grid.hy; s.hz = h->grid.hz;
+      s.a = h->geom.a; s.b = h->geom.b;
+      s.modes_m = h->geom.modes_m; s.modes_n = h->geom.modes_n;
+      s.igf = h->kind;
+      double* g = nullptr;
+      if ((e = cudaMalloc(&g, count * sizeof(double))) == cudaSuccess)
+        e = build_mode_spectrum(s, h->mxp, h->myp, h->fy, g, nullptr);
+      if (e == cudaSuccess) h->mgz64 = g;
+      else cudaFree(g);
+    }
+  }
+  if (e == cudaSuccess) e = cudaMemcpy(out, h->mgz64, count * sizeof(double), cudaMemcpyDeviceToHost);
   return status_of(e);
 }
 

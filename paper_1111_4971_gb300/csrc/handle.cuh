@@ -3,6 +3,8 @@
 
 #include <cuda_runtime.h>
 
+#include <mutex>
+
 #include "../../include/pipe_poisson.h"
 #include "modes_split.cuh"
 
@@ -63,6 +65,8 @@ struct pipe_handle {
   float *msx32 = nullptr, *msy32 = nullptr;
   double* mzp64 = nullptr;     // parameters of the z recurrences [mxp*myp][kModeZPar]
   float* mzp32 = nullptr;
+  double* mgz64 = nullptr;     // pipe_mode_spectrum's table, from its first call on
+  std::mutex mgz_mu;
   double* mkb64 = nullptr;     // banded operator in mode space: [mxp*myp][nb+1] real-space z kernel
   float* mkb32 = nullptr;
   // FP64: fragment tables of the split products (modes_split.cu), one allocation
