@@ -108,10 +108,11 @@ typedef struct pipe_handle pipe_handle;
  *    mode's column (Appendix A), and the back-projection.  Any mesh
  *    inside the pipe with nx and ny multiples of 16 (nx != ny allowed, up to
  *    4096 each), nz in {32, ..., 1024} as above, modes_m, modes_n <= 32;
- *    PIPE_F32 or PIPE_F64; not banded; and its kernels' shared memory within
- *    the device's 227 KB per CTA (it grows with ny and the modes: FP32 with
- *    20 x 20 modes takes ny up to about 1400, FP64 about 700; FP64 takes at
- *    most about 880 mode pairs, e.g. 32 x 24 but not 32 x 32).  Its tables
+ *    PIPE_F32 or PIPE_F64; full or banded; and, a rule on ny and the modes
+ *    that stands for itself (the kernels need less), a ring of field rows, the
+ *    y-mode table and 32 z values of modes_m*slots mode columns within 227 KB:
+ *    FP32 with 20 x 20 modes takes ny up to about 1400, FP64 about 700; FP64
+ *    takes at most about 880 mode pairs, e.g. 32 x 24 but not 32 x 32.  Its tables
  *    (FP64, with FP32 copies) take (nx*mxp + ny*myp + 12*mxp*myp)*12 bytes
  *    (FP64 about 10 times that, as fragments for the tensor cores) and its
  *    scratch (xblocks + 1)*mxp*myp*nz values of the dtype (the sizes of
@@ -242,7 +243,10 @@ int pipe_poisson_solve_host_stream(pipe_handle* h, const void* const* rho_host, 
  * choice and are capturable in a CUDA graph.  Results equal those of
  * pipe_poisson_solve up to rounding, and bitwise for FP32 handles whose plan is
  * z_warps = 16, z_pipe = 0, t_h = 1, t_threads = 512, and t_kind = 1 on
- * cell-centred meshes, 0 on others (the persistent kernel's shapes).
+ * cell-centred meshes, 0 on others (the persistent kernel's shapes).  A handle
+ * whose own form is the mode-space one (t_kind 3, the default of every FP64
+ * handle) runs transforms inside the persistent launch and the mode form
+ * outside it, so its last bits depend on the split that the timing picked.
  * Errors: PIPE_EINVAL (n < 1, null arrays), PIPE_EUNSUPPORTED (mixed dtypes
  * or devices), PIPE_ENOMEM, PIPE_ECUDA. */
 int pipe_poisson_solve_batched(pipe_handle* const* handles, const void* const* rho,
@@ -272,9 +276,8 @@ int pipe_batch_side_streams(pipe_handle* const* handles, int n, int* nside);
 int pipe_batch_select_streams(pipe_handle* const* handles, int n, int nside);
 
 /* Mode-form groups of the batched call: FP32 solves outside the persistent
- * launch that run the mode-space form with the occupancy-laid-out kernels
- * (pipe_get_plan t_kind 3 on a mesh symmetric in y, ny/2 in {16, 32, 64, 128})
- * and share nx, ny, nz, the mode counts and the y-mode table run together:
+ * launch that run the mode-space form (pipe_get_plan t_kind 3) and share nx, ny,
+ * nz, the mode counts and the mesh's symmetry in y run together:
  * one launch per stage for up to 64 solves, with the same kernels and the
  * same results, bit for bit, as their single-solve launches.  The tuner
  * times the call with and without them.  pipe_batch_grouped reports how

@@ -21,9 +21,9 @@
 //
 // The solves left outside the persistent launch run as their own launches,
 // on the caller's stream or dealt to side streams.  FP32 mode-space solves of
-// one shape among them can run as a group: one launch
-// per stage (projection, z convolution, back-projection) for up to 64 solves,
-// each CTA finding its solve from its block index.  A stage of many solves is
+// one shape among them can run as a group: one launch per stage (projection, z
+// convolution, back-projection) for up to 64 solves, each CTA finding its solve
+// from its block index.  A stage of many solves is
 // a grid of many waves, so the reduction phase of some CTAs overlaps the
 // field streams of others.  The tuner times the persistent/outside split, the
 // work-list order, the side streams and the grouping, and keeps the fastest.
@@ -513,9 +513,8 @@ static double spectrum_bytes(const pipe_handle* h) {
   return double(h->grid.nx) * h->grid.ny * (h->grid.nz + 1) * (h->grid.dtype == PIPE_F64 ? 16 : 8);
 }
 
-// the groups of a variant's outside solves: FP32 mode-form solves with the
-// of one shape, up to
-// kMaxModeGroup each; only groups of two or more are kept
+// the groups of a variant's outside solves: FP32 mode-form solves of one shape,
+// up to kMaxModeGroup each; only groups of two or more are kept
 static bool mode_groupable(const pipe_handle* h) {
   return h->grid.dtype == PIPE_F32 && h->use_modes && h->banded < 0;
 }

@@ -8,9 +8,10 @@ namespace pp {
 template <typename T>
 struct ModeArgs;
 
-// The mode form takes a mesh where these two are within a CTA's shared memory:
-// the sizes of a projection and a back-projection kernel that stage a ring of
-// field rows, the y-mode table and 32 z values of the mode columns.
+// The mode form takes a mesh where these two are within 227 KB: a ring of field
+// rows, the y-mode table and 32 z values of the mode columns.  A rule of the
+// interface, kept from kernels laid out so; the present ones need less (FP32:
+// modes_sums.cu reads a long y table through L1, FP64: modes_split.cu takes 64 KB).
 template <typename T>
 inline size_t mode_proj_smem(int ny, int mxp, int myp, bool fold) {
   constexpr int XB = sizeof(T) == 4 ? 16 : 8, ZC = 32;
@@ -55,9 +56,10 @@ inline int divisor_to_4(int n) {
 //   projection 7.2 / 7.3, back-projection 6.5 / 5.9 us; 128^2 x 1024, 8 / 4 / 16:
 //   20.3 / 21.9 / 31.6 and 17.5 / 18.1 / 17.1).  One x row a warp: 25.8 and 23.7.
 //   Groups: every x block its own while there are at most 16 (128^2 x 1024, 8 / 4
-//   groups: 20.3 / 23.5 us; all with x-mode sums of one slot at a time), else a divisor of 4 to 8: the partials (1.6 MB each
-//   at 400 columns of 1024) would come near the field's own bytes.  Their memory
-//   is at most 48 MiB, or what one partial per up to 4 blocks of 16 rows takes.
+//   groups: 20.3 / 23.5 us; all with x-mode sums of one slot at a time), else a
+//   divisor of 4 to 8: the partials (1.6 MB each at 400 columns of 1024) would
+//   come near the field's own bytes.  Their memory is at most 48 MiB, or what one
+//   partial per up to 4 blocks of 16 rows takes.
 constexpr int kModeRowsPerWarp = 2;
 struct ModeShape {
   int warps, reps, groups;

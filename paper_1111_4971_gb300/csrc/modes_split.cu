@@ -47,13 +47,17 @@
 // a plane's exponent go by a vote, and the warp's index is broadcast, so that what
 // follows from them stays in uniform registers (without: 105 us for the first).
 // Splitting costs some 45 integer instructions a value and putting an output
-// together some 30; they bound the two kernels (ALU pipe 48 and 55 % busy,
-// tensor pipe 21 and 38 %, DRAM 25 and 35 %, 11 warps an SM held to that by the
-// contraction's 96 accumulators).  128^2 x 1024, 20 x 20 modes, ncu, before ->
-// after: projection 516 -> 75 + 24 us (y, x), back-projection 468 -> 21 + 54 us;
-// the solve 1005 -> 180 us, and 256^2 x 512 with nodes on the wall (which now
-// folds too) 3230 -> 325 us.  Error against 64 bits over such meshes 4 to 8e-16,
-// the FP64 FMA sums' 4 to 9e-16.
+// together some 30.  No pipe is full (along y: ALU 51 and 53 % busy, issue 48 and
+// 51 %, tensor 22 and 38 %, DRAM 25 and 22 %): what bounds the kernels is latency,
+// with 11 warps an SM (the contraction's 96 accumulators) and 14.  128^2 x 1024, 20
+// x 20 modes, ncu, against FP64 FMAs: projection 516 -> 70 + 24 us (y, x),
+// back-projection 468 -> 21 + 54; the solve 1005 -> 162 us, and 256^2 x 512 with
+// nodes on the wall (which folds too) 3230 -> 284.
+// Error against 64 bits, relative L2: 4 to 5e-16 over such meshes, the FP64 FMA
+// sums' 4 to 7e-16.  Relative to the first row alone, for a bunch at the mesh's
+// centre, whose potential is small there: 3.2e-15 at 128 rows and 3.4e-15 at 512
+// (without the rows' scales 1.6e-14 and 6.9e-14, FMAs 0.7e-15 and 0.8e-15): an
+// entry far below its row's largest sine still has the row's cut.
 //
 // Values that are not finite give NaN in every output of their z plane (a stage
 // run by itself, pipe_stage_modes: of their 16 planes).
