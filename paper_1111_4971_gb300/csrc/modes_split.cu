@@ -638,7 +638,8 @@ __global__ void __launch_bounds__(32 * kSplitWarps, FOLD ? 4 : (KS == 2 ? 5 : 7)
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       const int r = 8 * tile + 2 * t + c;
-      const int x0 = e0.e20 - (c ? scale.y : scale.x), x1 = e1.e20 - (c ? scale.y : scale.x);
+      const unsigned sc = unsigned(c ? scale.y : scale.x);              // (wraps for a row of zeros, whose sums are 0)
+      const int x0 = int(unsigned(e0.e20) - sc), x1 = int(unsigned(e1.e20) - sc);
       const unsigned long long o0 = fixed(acc[0], c), o1 = fixed(acc[0], 2 + c);
       if constexpr (FOLD) {
         const unsigned long long v0 = fixed(acc[1], c), v1 = fixed(acc[1], 2 + c);
