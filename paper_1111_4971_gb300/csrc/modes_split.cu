@@ -42,8 +42,8 @@
 // sine is 0.005).  The expansion takes it off its output's exponent, the
 // contraction off the value's; a row that is zero, on the wall, takes no part in
 // the maxima.  Both together against one scale a tile: projection and
-// back-projection at 128^2 x 1024 90.5 + 70.9 -> 88.1 + 71.5 us, 256^2 x 512 on the
-// wall 190 + 128 -> 183 + 129, 48 x 80 x 512 21.4 + 18.4 -> 21.2 + 19.1: branches on
+// back-projection at 128^2 x 1024 90.5 + 70.9 -> 86.4 + 71.8 us, 256^2 x 512 on the
+// wall 190 + 128 -> 180 + 130, 48 x 80 x 512 21.4 + 18.4 -> 20.9 + 19.0: branches on
 // a plane's exponent go by a vote, and the warp's index is broadcast, so that what
 // follows from them stays in uniform registers (without: 105 us for the first).
 // Splitting costs some 45 integer instructions a value and putting an output
